@@ -103,17 +103,23 @@ typedef struct {
     void *cuda_stream;        /* cudaStream_t to run on; NULL: the context creates its own
                                  non-blocking stream (pass cudaStreamLegacy for the legacy
                                  default stream, whose handle is NULL) */
-    int time_block;           /* steps fused per launch (temporal blocking); <= 1: one.
-                                 D2Q5: 2, 4, 6, 8 or 16 with FP32 or BF16 storage (the fused
-                                 levels in between are FP32); D2Q9: 2 or 4 with FP32 storage */
+    int time_block;           /* steps fused per launch (temporal blocking): at most this many
+                                 at a time.  D2Q5: 2, 4, 6, 8 or 16 with FP32 or BF16 storage
+                                 (BF16: whole blocks, FP32 between their steps); D2Q9: 2 or 4
+                                 with FP32 storage.  <= 1: lb_step fuses steps by itself where
+                                 that is faster and changes nothing: with LB_STEP_AUTO, on 2-D
+                                 FP32 / BF16 grids without patch, slab or in-place streaming, the
+                                 results equal one launch per step bit for bit */
     /* Optional device allocator (e.g. PyTorch's caching allocator).  NULL: cudaMalloc. */
     void *(*dev_alloc)(size_t bytes, void *user);
     void (*dev_free)(void *ptr, void *user);
     void *alloc_user;
     int step_kernel;          /* LB_STEP_AUTO (0): the TMA-staged persistent step for 16-bit
                                  storage on rows of >= 1024 sites without a patch, the
-                                 register-streaming step otherwise; LB_STEP_DIRECT (1) / LB_STEP_STAGED
-                                 (2, no patch): always that step.  All give bit-identical results. */
+                                 register-streaming step otherwise, and several steps per launch
+                                 where that is faster (time_block); LB_STEP_DIRECT (1) /
+                                 LB_STEP_STAGED (2, no patch): always that step, one per launch.
+                                 All give bit-identical results. */
     int nz;                   /* planes of a 3-D grid (LB_D3Q7 only, BGK, no patch, no time
                                  blocking); <= 1: 2-D.  3-D arrays are [nz][ny][nx] (c_map,
                                  pressure) and [Q][nz][ny][nx] (state). */
@@ -291,15 +297,13 @@ typedef struct {
     size_t hbm_budget;       /* device bytes the server may hold; 0: 80% of free memory */
     int rounds_per_pass;     /* steps per scheduling pass between admission checks, >= 1 */
     int adjoint_workers;     /* threads running gradient sweeps, >= 1 */
-    int tb_min_ctas;         /* D2Q5 FP32/BF16 shots with no checkpoint or tape can advance
-                                4 steps per launch (a wavefront time-blocked batch).
-                                0: they do, with the rows per CTA (at most 64) that fill
-                                one wave of the GPU, when that is at least 12 rows and
-                                their states outgrow three quarters of L2 (a few small
-                                shots step one launch at a time).  > 0: they do, at
-                                64 rows per CTA, when together they make at least this
-                                many CTAs.  < 0: never.  Both forms give the same results
-                                to FP32 rounding. */
+    int tb_min_ctas;         /* D2Q5 shots (FP32 with no checkpoint; BF16 also with no tape) can
+                                advance 4 steps per launch.  0: they do.  > 0: they do, at
+                                64 rows per warp, when together they make at least this many
+                                CTAs.  < 0: never.  FP32 results are the same bit for bit; so
+                                are BF16 results, except that BF16 shots keep FP32 between the
+                                4 steps of a launch with tb_min_ctas > 0, or with 0 while the
+                                ready shots together outgrow three quarters of L2. */
 } lb_server_config;
 
 typedef struct {

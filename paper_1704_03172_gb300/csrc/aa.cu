@@ -244,7 +244,7 @@ lb_status aa_step(lb_ctx *ctx, int n) {
         a.trace_row = (ctx->trace && row >= 0 && row < ctx->trace_cap)
                           ? ctx->trace + row * ctx->nrec
                           : nullptr;
-        AaRec r{a.trace_row ? ctx->tb5_off : nullptr, ctx->tb5_x, ctx->tb5_id};
+        AaRec r{a.trace_row ? ctx->row_off : nullptr, ctx->row_x, ctx->row_id};
         if (ctx->staged) {  // BF16 on wide rows: the TMA-staged persistent form
             lb_status st = stream_launch_aa(ctx, a, ex, r.row_off, r.rec_x, r.rec_id);
             if (st != LB_OK) return st;

@@ -10,7 +10,7 @@ namespace lbaa {
 
 using namespace lbk;
 
-struct AaRec {           // receivers by row, x ascending (tb5_set_receivers' lists)
+struct AaRec {           // receivers by row, x ascending (wave_set_receivers' lists)
     const int *row_off;  // [ny + 1], or nullptr: no receivers this step
     const int *rec_x;
     const int *rec_id;

@@ -646,15 +646,15 @@ extern "C" lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *g
     const int adj_blocks = (int)(((long long)ctx->ny * segs4 + kWarps - 1) / kWarps);
     // replay steps t = from .. from + n - 1 starting at state `in`; the state after the
     // last one goes to `last` (when given); rho(t) goes to tape[t - from] (when given).
-    // FP32 contexts replay K steps per launch with the time-blocked kernel wherever a whole
-    // block of K fits (not from a raw state); other steps run one per launch.
-    const int K = ctx->cfg.storage == LB_F32 ? (ctx->Q == 5 ? 8 : ctx->Q == 9 ? 4 : 0) : 0;
+    // Several steps per launch where the fused kernel has them (not from a raw state): its
+    // results are the one-step kernels', so a BF16 replay reproduces the forward run.
+    const bool fuse = wave_supported(ctx) && wave_pays(ctx);
     lb_status rst = LB_OK;
     auto replay = [&](const void *in, bool raw, long long from, int n, void *last, bool record) {
         int x = 0;
         for (int m = 0; m < n;) {
             const bool first_raw = raw && m == 0;
-            const int len = (K > 0 && !first_raw && n - m >= K) ? K : 1;
+            const int len = fuse && !first_raw ? wave_steps(ctx, n - m) : 1;
             StepArgs a = base;
             a.in = in;
             a.out = (m + len == n && last) ? last : X[x];
@@ -663,7 +663,7 @@ extern "C" lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *g
             a.rho_out = record ? tape + (size_t)m * plane : nullptr;
             a.rho_stride = (long long)plane;
             if (len > 1) {
-                if (rst == LB_OK) rst = tb_launch_args(ctx, a, len);
+                if (rst == LB_OK) rst = wave_launch_args(ctx, a, len);
             } else if (ctx->staged) {
                 stream_launch(ctx, a, 0);  // cannot fail once the forward run has stepped
             } else {

@@ -40,11 +40,10 @@ struct lb_ctx {
     float *rho_tape = nullptr;      // lb_record_rho: rho(t) [tape_cap][ny][pitch] from tape_t0
     long long tape_t0 = 0;
     int tape_cap = 0;
-    int *tb_off = nullptr;          // temporal blocking: per-tile receiver list offsets
-    int *tb_rec = nullptr;          // receiver indices grouped by tile
-    int *tb5_off = nullptr;         // D2Q5 wavefront blocking: per-row receiver offsets [ny + 2]
-    int *tb5_x = nullptr;           // their x (ascending within a row)
-    int *tb5_id = nullptr;          // their receiver index
+    int *row_off = nullptr;         // receivers by row (one allocation): offsets [ny + 2],
+    int *row_x = nullptr;           // their x (ascending within a row)
+    int *row_id = nullptr;          // their receiver index
+    int *row_y = nullptr;           // their row
     bool ckpt_raw0 = false;         // raw flag of the time-0 checkpoint
     float *src_tab = nullptr;
     int src_nt = 0, src_x = 0, src_y = 0;
@@ -151,37 +150,43 @@ void ckpt_reset(lb_ctx *ctx);
 void tape_reset(lb_ctx *ctx);
 float *tape_row(const lb_ctx *ctx, long long t);
 
-// temporal blocking (tblock.cu)
+// several steps per launch (wave.cu): the cfg.time_block values, and K steps of a context
 bool tb_supported(int Q, int K);
 // TMA-staged persistent step (stream_step.cu): one LB step of the context's grid
 lb_status stream_launch(lb_ctx *ctx, const lbk::StepArgs &a, int rec_blocks);
 // its in-place form (BF16, D2Q5 / D2Q9): the site-local step, or the exchange step; receivers
-// from the per-row lists of tb5_set_receivers (rec_off nullptr: none this step)
+// from the per-row lists of wave_set_receivers (rec_off nullptr: none this step)
 lb_status stream_launch_aa(lb_ctx *ctx, const lbk::StepArgs &a, bool exchange, const int *rec_off,
                            const int *rec_x, const int *rec_id);
-lb_status tb_set_receivers(lb_ctx *ctx, const int *xy, int nrec);
 lb_status tb_launch(lb_ctx *ctx, int K);
-lb_status tb_launch_args(lb_ctx *ctx, const lbk::StepArgs &a, int K);
 // in-place streaming (aa.cu): n steps of an LB_STREAM_AA context
 lb_status aa_step(lb_ctx *ctx, int n);
-// D2Q5 wavefront temporal blocking (tblock5.cu)
-bool tb5_supported(int K);
-lb_status tb5_set_receivers(lb_ctx *ctx, const int *xy, int nrec);
+// warp wavefront (wave.cu): 2, 4 or 6 steps of a D2Q5, 2 or 4 of a D2Q9 grid per launch, FP32 or
+// BF16 storage, with the one-step kernels' results bit for bit.  Whether a context has it, whether
+// it pays without being asked for, the steps the next launch takes of n wanted, the receivers' row
+// lists, and the launch
+bool wave_supported(const lb_ctx *ctx);
+bool wave_pays(const lb_ctx *ctx);
+int wave_steps(const lb_ctx *ctx, int n);
+lb_status wave_set_receivers(lb_ctx *ctx, const int *xy, int nrec);
+lb_status wave_launch_args(lb_ctx *ctx, const lbk::StepArgs &a, int K);
+// its served batches of D2Q5 shots, kServeSteps steps per launch: staging bytes of one launch's
+// descriptors, whether a shot can take the steps now, the rows per warp that suit n shots
+// together, a shot's CTAs at H rows per warp, the fill (advancing the shots) and the launch from
+// the device copy of the staging block.  BF16 shots round at every step, as the one-step
+// kernels do, while the shots in hand are few; once they fill a wave of 12 rows x 248 columns
+// per CTA slot and outgrow three quarters of L2 they keep FP32 between the steps of a launch.
+constexpr int kServeSteps = 4;
+size_t wave_batch_bytes(int n);
+bool wave_batch_ready(const lb_ctx *ctx);
+int wave_batch_rows(lb_ctx *const *ctxs, int n);
+bool wave_batch_round(lb_ctx *const *ctxs, int n);
+int wave_batch_blocks(const lb_ctx *ctx, int H);
+int wave_batch_fill(lb_ctx *const *ctxs, int n, int H, void *h);
+cudaError_t wave_batch_launch(const void *d, int n, int blocks, bool mrt, int storage, bool round,
+                              cudaStream_t stream);
+// D2Q5 BF16 blocks of cfg.time_block steps with FP32 between them (tblock5.cu)
 lb_status tb5_launch_args(lb_ctx *ctx, const lbk::StepArgs &a, int K);
-// served batches of D2Q5 shots, K = kServeTb steps per launch (tblock5.cu; 4: the fastest
-// wavefront depth, 3 CTAs per SM at 72 registers): staging bytes of one
-// launch's descriptors, whether a shot can take K steps now, its strips and its CTAs at H
-// output rows per CTA, the CTAs one wave of the batched kernel holds on the current device,
-// the fill (advancing the shots) and the launch from the device copy of the staging block
-constexpr int kServeTb = 4;
-size_t tb5_batch_bytes(int n);
-bool tb5_batch_ready(const lb_ctx *ctx, int K);
-int tb5_strips(const lb_ctx *ctx, int K);
-int tb5_batch_blocks(const lb_ctx *ctx, int K, int H);
-int tb5_batch_wave(int K);
-int tb5_batch_fill(lb_ctx *const *ctxs, int n, int K, int H, void *h);
-cudaError_t tb5_batch_launch(const void *d, int n, int K, int blocks, bool mrt, bool per,
-                             int storage, cudaStream_t stream);
 
 // test-only FP64 storage (f64.cu): medium and coefficients, source table, steps, and the
 // state transforms (mode 0 pressure, 1 populations; FP32 arrays f or FP64 arrays d)

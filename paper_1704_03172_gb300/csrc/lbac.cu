@@ -489,7 +489,8 @@ lb_status lb_footprint(const lb_config *cfg, int nt, int nrec, int want_adjoint,
     const size_t nbuf = cfg->streaming == LB_STREAM_AA ? 1 : 2;
     size_t b = nbuf * q * plane * elem_bytes(cfg->storage) + plane * 4 + plane + 1024;
     if (cfg->storage == LB_F64) b += plane * 8 + (size_t)std::max(nt, 0) * 8 + 256;
-    if (nrec > 0 && nt > 0) b += (size_t)nt * nrec * 4 + (size_t)nrec * 8;
+    if (nrec > 0 && nt > 0)
+        b += (size_t)nt * nrec * 4 + (size_t)nrec * 16 + (size_t)std::max(cfg->ny, 1) * 4 + 256;
     if (nt > 0) b += (size_t)nt * 4;
     // refinement levels (refine.cu): per patch, two population buffers with a ghost ring and
     // its eta^2 plane, the interface lists and three snapshot slots, the nested patch's
@@ -793,8 +794,8 @@ static lb_status set_receivers_rows(lb_ctx *ctx, const int *xy, int nrec, int nt
     ctx->rec_xy.assign(xy, xy + 2 * (size_t)nrec);
     ctx->trace_cap = nt_capacity;
     if (ctx->refined) return refine_set_receivers(ctx, xy, nrec);
-    if (ctx->aa) return tb5_set_receivers(ctx, xy, nrec);  // rows of receivers, x ascending
-    if (ctx->cfg.time_block > 1) return tb_set_receivers(ctx, xy, nrec);
+    // rows of receivers, x ascending: the in-place and the fused steps record from them
+    if (ctx->aa || wave_supported(ctx)) return wave_set_receivers(ctx, xy, nrec);
     return LB_OK;
 }
 
@@ -1029,6 +1030,27 @@ lb_status lb_step(lb_ctx *ctx, int n) {
     return LB_OK;
 }
 
+// Steps of the next launch, of which `left` are wanted: several where a fused kernel takes
+// them, never across a checkpoint time, the end of the trace buffer or of the rho tape (single
+// steps keep all three exact), and one from a raw state.
+static int fused_steps(const lb_ctx *ctx, int left) {
+    const int T = ctx->cfg.time_block;
+    if (ctx->raw || left < 2) return 1;
+    long long room = left;
+    if (ctx->ckpt_every > 0)
+        room = std::min<long long>(room, ctx->ckpt_every - (ctx->t - ctx->ckpt_t0) % ctx->ckpt_every);
+    const long long row = ctx->t - ctx->t_rec0;
+    if (ctx->trace && row < ctx->trace_cap) room = std::min<long long>(room, ctx->trace_cap - row);
+    const long long trow = ctx->t - ctx->tape_t0;
+    const bool taping = ctx->rho_tape && trow < ctx->tape_cap;
+    if (taping) room = std::min<long long>(room, ctx->tape_cap - trow);
+    if (T > 1 && ctx->cfg.storage == LB_BF16)  // FP32 between the levels: no rho record
+        return room >= T && !taping ? T : 1;
+    if (T > 1) return wave_steps(ctx, (int)std::min<long long>(room, T));
+    if (ctx->cfg.step_kernel != LB_STEP_AUTO || !wave_supported(ctx) || !wave_pays(ctx)) return 1;
+    return wave_steps(ctx, (int)std::min<long long>(room, 1 << 20));
+}
+
 static lb_status step_n(lb_ctx *ctx, int n) {
     if (ctx->refined) return refine_step(ctx, n);
     if (ctx->cfg.storage == LB_F64) return f64_step(ctx, n);
@@ -1038,35 +1060,15 @@ static lb_status step_n(lb_ctx *ctx, int n) {
     }
     StepFn fn = pick_step(ctx);
     StepArgs a = base_args(ctx);
-    const int K = ctx->cfg.time_block;
     for (int k = 0; k < n;) {
         if (ctx->ckpt_every > 0) {
             lb_status st = ckpt_maybe_save(ctx);
             if (st != LB_OK) return st;
         }
-        if (K > 1 && n - k >= K && !ctx->raw) {
-            // K fused steps, unless they would straddle a checkpoint time or the end
-            // of the trace capacity; then single steps keep both exact
-            const long long row = ctx->t - ctx->t_rec0;
-            const bool straddle_ckpt =
-                ctx->ckpt_every > 0 && (ctx->t - ctx->ckpt_t0) % ctx->ckpt_every + K > ctx->ckpt_every;
-            const bool straddle_trace =
-                ctx->trace && row < ctx->trace_cap && row + K > ctx->trace_cap;
-            const long long trow = ctx->t - ctx->tape_t0;
-            // the time-blocked kernel records the rho tape for FP32 storage only
-            const bool straddle_tape =
-                ctx->rho_tape && trow < ctx->tape_cap &&
-                (trow + K > ctx->tape_cap || ctx->cfg.storage != LB_F32);
-            if (!straddle_ckpt && !straddle_trace && !straddle_tape) {
-                lb_status st = tb_launch(ctx, K);
-                if (st != LB_OK) return st;
-                k += K;
-                continue;
-            }
-        }
-        lb_status st = launch_step(ctx, fn, a);
+        const int K = fused_steps(ctx, n - k);
+        lb_status st = K > 1 ? tb_launch(ctx, K) : launch_step(ctx, fn, a);
         if (st != LB_OK) return st;
-        k += 1;
+        k += K;
     }
     return check_launch(ctx, "step_kernel");
 }

@@ -11,9 +11,9 @@
 //              reading its own StepArgs descriptor (uploaded once per pass), so
 //              many small shots share one launch and fill the GPU together.  D2Q5
 //              FP32 / BF16 shots that are far enough from their end take their steps
-//              kServeTb at a time instead: one time-blocked launch
-//              (tb5_batch_kernel, tblock5.cu) per group advances every such shot by
-//              kServeTb steps.
+//              kServeSteps at a time instead: one launch of the warp wavefront
+//              (wave_batch_kernel, wave.cuh) per group advances every such shot by
+//              kServeSteps steps.
 //              Shots that finish leave the batch (their traces are copied to
 //              pinned host memory), shots that are ready join at the next pass;
 //   workers    run the adjoint of gradient requests (lb_adjoint) on their own
@@ -140,8 +140,6 @@ struct lb_server {
     size_t cap = 0;
     void *d_tb = nullptr, *h_tb = nullptr;  // time-blocked launches' descriptor blocks
     size_t tb_cap = 0;
-    int tb_wave = 0;  // CTAs one wave of the time-blocked batch kernel holds (0: not asked yet)
-    long long l2_bytes = -1;  // the device's L2 size (-1: not asked yet)
     cudaEvent_t staged = nullptr;
     std::mutex pin_mu;
     std::multimap<size_t, void *> pinned;  // free pinned trace buffers by size
@@ -253,9 +251,6 @@ void admit(lb_server *S, Req *r) {
     if (st == LB_OK && !r->wav.empty())
         st = lb_set_source(ctx, r->src_x, r->src_y, r->wav.data(), (int)r->wav.size());
     if (st == LB_OK) st = lb_set_receivers(ctx, r->rec.data(), (int)r->rec.size() / 2, r->nt);
-    if (st == LB_OK && c.lattice == LB_D2Q5 && (c.storage == LB_F32 || c.storage == LB_BF16) &&
-        !r->rec.empty())  // the receiver rows of the time-blocked batches
-        st = tb5_set_receivers(ctx, r->rec.data(), (int)r->rec.size() / 2);
     if (st == LB_OK) st = lb_init_pressure(ctx, nullptr, 0);
     if (st == LB_OK && r->want_grad)
         st = r->tape ? lb_record_rho(ctx, r->nt) : lb_checkpoint_every(ctx, r->ckpt);
@@ -365,53 +360,31 @@ void pass(lb_server *S) {
     };
     // wait until the previous pass has consumed the staging buffers
     if (S->staged) cudaEventSynchronize(S->staged);
-    // shots that take this pass's steps K at a time: one time-blocked launch per group and
-    // block of K steps
-    const int KB = kServeTb, nblk = R / KB;
-    // Shots that take this pass's steps K at a time.  A wavefront CTA sweeps its rows one
-    // after another, so the launch must fill a wave of CTAs with chunks tall enough that
-    // the 2K warm-up rows of each cost little.  By default (tb_min_ctas = 0) the pass takes
-    // the chunk height (at most 16K rows) that fills one wave with every ready shot: at
-    // least 3K rows, and states larger than L2 can hold, else none of them blocks this pass
-    // (two-layer 1024^2 alone, K = 8: 112 GLUPS blocked with one-wave chunks of 18 rows
-    // against 153 one step per launch; 4096^2: 295 against 160).  All CTAs of the launch
-    // then sweep about the same number of rows, whatever their shot's size.  With
-    // tb_min_ctas > 0 the shots block at 16K rows when together they make that many CTAs;
-    // below 0 never.
+    // Shots that take this pass's steps K at a time (wave.cuh): one launch per group and block of
+    // K steps.  By default (tb_min_ctas = 0) every ready shot does, at the rows per warp that
+    // suit them together: even a lone 256^2 shot runs faster so (2.7 against 3.4 us a step).
+    // With tb_min_ctas > 0 they do at 16K rows when together they make that many CTAs; below 0
+    // never.
+    const int KB = kServeSteps, nblk = R / KB;
     std::vector<Req *> tbs, rest;
-    const int H16 = 16 * KB;
-    int tb_rows = H16;
+    std::vector<lb_ctx *> cs;
+    int tb_rows = 16 * KB;
+    bool round = false;  // BF16 shots: at every step (wave_batch_round)
     for (Req *r : batched) {
         const bool ok = S->cfg.tb_min_ctas >= 0 && nblk > 0 && r->nt - r->steps >= nblk * KB &&
-                        tb5_batch_ready(r->ctx, KB);
+                        wave_batch_ready(r->ctx);
         (ok ? tbs : rest).push_back(r);
     }
     if (!tbs.empty()) {
         bool use = true;
         if (S->cfg.tb_min_ctas > 0) {
             long long ctas = 0;
-            for (Req *r : tbs) ctas += tb5_batch_blocks(r->ctx, KB, H16);
+            for (Req *r : tbs) ctas += wave_batch_blocks(r->ctx, tb_rows);
             use = ctas >= S->cfg.tb_min_ctas;
-        } else {  // the chunk height that fills one wave
-            if (S->tb_wave == 0) S->tb_wave = tb5_batch_wave(KB);
-            if (S->l2_bytes < 0) {
-                int v = 0;
-                if (cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, S->device) != cudaSuccess) {
-                    cudaGetLastError();  // this query's own failure: assume no L2
-                    v = 0;
-                }
-                S->l2_bytes = v;
-            }
-            long long rows = 0, state = 0;  // sums over the shots of strips x rows, state bytes
-            for (Req *r : tbs) {
-                rows += (long long)tb5_strips(r->ctx, KB) * r->ctx->ny;
-                state += 2LL * r->ctx->Q * r->ctx->ny * r->ctx->pitch * r->ctx->ebytes;
-            }
-            const long long h = (rows + S->tb_wave - 1) / S->tb_wave;
-            tb_rows = (int)std::min<long long>(H16, h);
-            // blocking saves HBM traffic; states that fit in three quarters of L2 have none
-            // to save (32 shots of 256^2, 84 MB: 3.7x over one by one stepped, 3.0x blocked)
-            use = tb_rows >= 3 * KB && 4 * state > 3 * S->l2_bytes;
+        } else {
+            for (Req *r : tbs) cs.push_back(r->ctx);
+            tb_rows = wave_batch_rows(cs.data(), (int)cs.size());
+            round = wave_batch_round(cs.data(), (int)cs.size());
         }
         if (!use) {
             rest.insert(rest.end(), tbs.begin(), tbs.end());
@@ -424,7 +397,7 @@ void pass(lb_server *S) {
     struct TbLaunch {
         size_t off;
         int n, blocks;
-        bool mrt, per;
+        bool mrt;
         int storage;
         size_t g0, g1;
     };
@@ -434,7 +407,7 @@ void pass(lb_server *S) {
         for (size_t g0 = 0; g0 < tbs.size();) {  // staging bytes of every launch
             size_t g1 = g0;
             while (g1 < tbs.size() && key(tbs[g1]) == key(tbs[g0])) g1++;
-            tb_bytes += nblk * tb5_batch_bytes((int)(g1 - g0));
+            tb_bytes += nblk * wave_batch_bytes((int)(g1 - g0));
             g0 = g1;
         }
         if (!ensure_tb_capacity(S, tb_bytes)) {
@@ -444,7 +417,6 @@ void pass(lb_server *S) {
             tbs.clear();
         }
         size_t off = 0;
-        std::vector<lb_ctx *> cs;
         for (int j = 0; j < nblk && !tbs.empty(); j++) {
             for (size_t g0 = 0; g0 < tbs.size();) {
                 size_t g1 = g0;
@@ -453,11 +425,10 @@ void pass(lb_server *S) {
                 for (size_t q = g0; q < g1; q++) cs.push_back(tbs[q]->ctx);
                 const int n = (int)(g1 - g0);
                 const int blocks =
-                    tb5_batch_fill(cs.data(), n, KB, tb_rows, static_cast<char *>(S->h_tb) + off);
+                    wave_batch_fill(cs.data(), n, tb_rows, static_cast<char *>(S->h_tb) + off);
                 const lb_config &c0 = tbs[g0]->cfg;
-                tb_launches.push_back({off, n, blocks, c0.collision == LB_MRT,
-                                       c0.boundary == LB_PERIODIC, c0.storage, g0, g1});
-                off += tb5_batch_bytes(n);
+                tb_launches.push_back({off, n, blocks, c0.collision == LB_MRT, c0.storage, g0, g1});
+                off += wave_batch_bytes(n);
                 g0 = g1;
             }
             for (Req *r : tbs) r->steps += KB;
@@ -538,8 +509,8 @@ void pass(lb_server *S) {
         return;
     }
     for (const TbLaunch &L : tb_launches) {  // time-blocked blocks of K steps
-        e = tb5_batch_launch(static_cast<char *>(S->d_tb) + L.off, L.n, KB, L.blocks, L.mrt, L.per,
-                             L.storage, S->stream);
+        e = wave_batch_launch(static_cast<char *>(S->d_tb) + L.off, L.n, L.blocks, L.mrt, L.storage,
+                              round, S->stream);
         if (e != cudaSuccess) {
             const std::string msg = std::string("time-blocked batch: ") + cudaGetErrorString(e);
             set_err(S, msg);

@@ -330,53 +330,9 @@ __global__ void __launch_bounds__(kWS, tb5_min_blocks<K>()) tb5_kernel(const Ste
     tb5_body<MRT, K, REC, ST>(a, tb, blockIdx.x, blockIdx.y, xs_mem, s_tab);
 }
 
-// Several independent grids ("shots") advanced by K steps in one launch: shot k owns
-// blocks [first[k], first[k + 1]) of the grid, laid out as its strips x row chunks, and
-// reads its own descriptors (the served batches; no rho tape).
-template <bool MRT, int K, typename ST>
-__global__ void __launch_bounds__(kWS, tb5_min_blocks<K>())
-    tb5_batch_kernel(const StepArgs *__restrict__ args, const Tb5Args *__restrict__ tbs,
-                     const int *__restrict__ strips, const int *__restrict__ first, int nshots) {
-    pdl_trigger_and_wait();
-    extern __shared__ float xs_mem[];
-    __shared__ float s_tab[kWS];
-    __shared__ StepArgs sa;
-    __shared__ Tb5Args stb;
-    __shared__ int s_blk, s_strips;
-    if (threadIdx.x == 0) {
-        int lo = 0, hi = nshots - 1;  // shot with first[k] <= blockIdx.x < first[k + 1]
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (first[mid] <= (int)blockIdx.x)
-                lo = mid;
-            else
-                hi = mid - 1;
-        }
-        sa = args[lo];
-        stb = tbs[lo];
-        s_strips = strips[lo];
-        s_blk = (int)blockIdx.x - first[lo];
-    }
-    __syncthreads();
-    const int blk = s_blk, ns = s_strips;
-    tb5_body<MRT, K, false, ST>(sa, stb, blk % ns, blk / ns, xs_mem, s_tab);
-}
-
-
 using Tb5Fn = void (*)(const StepArgs, const Tb5Args);
-using Tb5BatchFn = void (*)(const StepArgs *, const Tb5Args *, const int *, const int *, int);
 
-// one storage type's kernels (tblock5.cu: FP32, tblock5_bf16.cu: BF16); nullptr where absent
-Tb5Fn pick_f32(int K, bool mrt, bool rec);
-Tb5Fn pick_bf16(int K, bool mrt, bool rec);
-Tb5BatchFn pick_batch_f32(int K, bool mrt);
-Tb5BatchFn pick_batch_bf16(int K, bool mrt);
-
-template <int K, typename ST, bool WITH_REC = true> Tb5Fn pick_k(bool mrt, bool rec) {
-    if constexpr (WITH_REC) {
-        if (rec) return mrt ? tb5_kernel<true, K, true, ST> : tb5_kernel<false, K, true, ST>;
-    }
-    if (rec) return nullptr;
+template <int K, typename ST> Tb5Fn pick_k(bool mrt) {
     return mrt ? tb5_kernel<true, K, false, ST> : tb5_kernel<false, K, false, ST>;
 }
 

@@ -1,0 +1,345 @@
+// wave.cu -- host side of the warp wavefront (kernels: wave.cuh): FP32 D2Q5 instances, the
+// choice of steps per launch and of the launch shape, receiver row lists and served batches.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <atomic>
+#include <vector>
+
+#include "lb_kernels.cuh"
+#include "lb_runtime.h"
+#include "wave.cuh"
+#include "wave_host.h"
+
+using namespace lbk;
+using namespace lbrt;
+using namespace lbwave;
+
+namespace lbwave {
+WavePick pick_d2q5_f32(int ck, int K, bool rec) {
+    if (K == 6)  // BGK only (wave_steps)
+        return ck == kLossless ? rec ? pick_one<5, kLossless, 6, true, float, false>()
+                                     : pick_one<5, kLossless, 6, false, float, false>()
+                               : rec ? pick_one<5, kBgk, 6, true, float, false>()
+                                     : pick_one<5, kBgk, 6, false, float, false>();
+    return K == 4 ? pick_rec<5, 4, float, false>(ck, rec) : pick_rec<5, 2, float, false>(ck, rec);
+}
+WaveBatchPick pick_batch_f32(bool mrt) { return pick_batch<float, false>(mrt); }
+}  // namespace lbwave
+
+namespace {
+
+int collision_kind(const lb_ctx *c) {
+    if (c->cfg.collision == LB_MRT) return kMrt;
+    return c->Q == 5 && (float)(1.0 / c->cfg.tau) == 2.f ? kLossless : kBgk;
+}
+
+WavePick pick(const lb_ctx *c, int K, bool rec) {
+    const int ck = collision_kind(c);
+    if (c->Q == 9)
+        return c->cfg.storage == LB_BF16 ? pick_d2q9_bf16(ck, K, rec) : pick_d2q9_f32(ck, K, rec);
+    return c->cfg.storage == LB_BF16 ? pick_d2q5_bf16(ck, K, rec) : pick_d2q5_f32(ck, K, rec);
+}
+
+int sm_count() {
+    static std::atomic<int> sms{0};
+    int v = sms.load(std::memory_order_relaxed);
+    if (!v) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            v = 1;
+        }
+        sms.store(v, std::memory_order_relaxed);
+    }
+    return v;
+}
+
+// What a row in the sponge counts against kInner: an iteration with sponge factors issues half as
+// many instructions again.  The four-step FP32 BGK launch waits for HBM in part and hides some
+// of that: 4/3 there (4096^2: 514 GLUPS against 496), 3/2 elsewhere (MRT: 525 against 451, six
+// steps: 570 against 546).
+int outer_weight(const lb_ctx *c, int K) {
+    return c->Q == 5 && K <= 4 && c->cfg.storage == LB_F32 && c->cfg.collision == LB_BGK ? 8 : 9;
+}
+
+// Strips, and which of them meet the sponge or a face.  Strip b takes columns b out - halo ..
+// b out - halo + kCols - 1, recomputed ones included.
+void strips_of(WaveArgs &w, int nx, int K, int sponge, bool per) {
+    const int out = out_cols(K);
+    w.per = per ? 1 : 0;
+    w.strips = (nx + out - 1) / out;
+    w.edge_l = w.edge_r = 0;
+    if (!per || sponge > 0 || nx % 2) {
+        w.edge_l = std::min(w.strips, (sponge + halo(K) + out - 1) / out);
+        const int first = std::max(0, nx - sponge - (kCols - halo(K)) + out) / out;
+        w.edge_r = w.strips - std::min(w.strips, std::max(w.edge_l, first));
+    }
+}
+
+// n row chunks for the inner strips; returns the tasks
+long long set_chunks(WaveArgs &w, int ny, long long n) {
+    const int edge = w.edge_l + w.edge_r;
+    w.chunks = (int)n;
+    w.chunks_e = (int)std::min<long long>(ny, (w.outer * n + kInner - 1) / kInner);
+    const long long t = (long long)(w.strips - edge) * w.chunks + (long long)edge * w.chunks_e;
+    w.tasks = (int)t;
+    return t;
+}
+
+// Row chunks of a grid.  A warp sweeps its H + 2K rows one after another, of which 2K are
+// recomputed, so few tall chunks waste little and many short ones finish sooner while warps are
+// missing.  With m warps per scheduler an iteration of all of them takes about (4 + m) x 0.12 us
+// (K = 4, GB300: 0.57, 0.67, 0.82 and 0.96 us for m = 1 .. 4 at 4096^2, 0.66 .. 1.0 at 512^2);
+// the m that makes (H + 2K)(4 + m) smallest wins, and its tasks fit one wave.
+void shape(WaveArgs &w, int ny, int K, int max_m) {
+    const long long slots1 = (long long)sm_count() * kWarpsPerCta;
+    long long cost = -1, best = 1;
+    for (int m = 1; m <= max_m; m++) {
+        long long n = std::max<long long>(1, std::min<long long>(ny, m * slots1 / w.strips));
+        while (n > 1 && set_chunks(w, ny, n) > m * slots1) n--;
+        const long long c = ((ny + n - 1) / n + 2 * K) * (4 + m);
+        if (cost < 0 || c < cost) cost = c, best = n;
+    }
+    set_chunks(w, ny, best);
+}
+
+}  // namespace
+
+bool wave_supported(const lb_ctx *c) {
+    return (c->Q == 5 || c->Q == 9) && c->nz <= 1 && !c->refined && !c->aa && !c->slab_nyg &&
+           (c->cfg.storage == LB_F32 || c->cfg.storage == LB_BF16);
+}
+
+// A launch of four steps takes about 10 us however small the grid is, and longer with receivers;
+// a step alone takes 3 (128^2: 3.5 us a step fused against 3.0; 512^2: 4.6 against 5.4).
+bool wave_pays(const lb_ctx *c) { return (long long)c->ny * c->pitch >= (128LL << 10); }
+
+// Six steps (three CTAs per SM) beat four (four CTAs) where HBM is the limit: FP32 BGK grids well
+// beyond L2 (8192^2: 645 GLUPS against 560, 3000 x 2500: 470 against 440; 2048^2, 168 MB: 379
+// against 388).  MRT and BF16 are bound by issue first and run four (4096^2 MRT: 525 against
+// 470, BF16: 541 against 493).
+int wave_steps(const lb_ctx *c, int n) {
+    if (c->Q == 5 && c->cfg.storage == LB_F32 && c->cfg.collision == LB_BGK && n >= 6 && n != 8 &&
+        2LL * 5 * 4 * c->ny * c->pitch >= (200LL << 20))
+        return 6;
+    // D2Q9 BF16: four steps on large grids, two on small ones (4096^2: 261 against 229 GLUPS,
+    // 2048^2: 192 against 198, 512^2: 46 against 54); FP32: four (4096^2: 264 against 165)
+    if (c->Q == 9 && c->cfg.storage == LB_BF16 && (long long)c->ny * c->pitch < (6LL << 20))
+        return n >= 2 ? 2 : 1;
+    return n >= 4 ? 4 : n >= 2 ? 2 : 1;
+}
+
+// Per-row receiver lists (rows of the context, x ascending), one allocation.
+lb_status wave_set_receivers(lb_ctx *ctx, const int *xy, int nrec) {
+    if (ctx->row_off) dev_free(ctx, ctx->row_off);
+    ctx->row_off = ctx->row_x = ctx->row_id = ctx->row_y = nullptr;
+    const size_t no = (size_t)ctx->ny + 2, nr = (size_t)std::max(nrec, 1);
+    std::vector<int> all(no + 3 * nr, 0);
+    int *off = all.data(), *xs = off + no, *ids = xs + nr, *ys = ids + nr;
+    for (int r = 0; r < nrec; r++) off[(size_t)xy[2 * r + 1] + 1]++;
+    for (size_t k = 1; k < no; k++) off[k] += off[k - 1];
+    for (int r = 0; r < nrec; r++) ids[r] = r;
+    std::stable_sort(ids, ids + nrec, [&](int p, int q) {
+        return xy[2 * p + 1] != xy[2 * q + 1] ? xy[2 * p + 1] < xy[2 * q + 1] : xy[2 * p] < xy[2 * q];
+    });
+    for (int k = 0; k < nrec; k++) xs[k] = xy[2 * ids[k]], ys[k] = xy[2 * ids[k] + 1];
+    int *d = static_cast<int *>(dev_alloc(ctx, all.size() * sizeof(int)));
+    if (!d) return fail(ctx, LB_ENOMEM, "row receiver lists");
+    cudaError_t e = cudaMemcpyAsync(d, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice,
+                                    ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);  // `all` goes out of scope
+    ctx->row_off = d;
+    ctx->row_x = d + no;
+    ctx->row_id = ctx->row_x + nr;
+    ctx->row_y = ctx->row_id + nr;
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "row receiver lists");
+    return LB_OK;
+}
+
+// K fused steps with the caller's arguments (a.in must not be raw); receivers when
+// a.trace_row is set and the row lists exist; rho of every level when a.rho_out is set.
+lb_status wave_launch_args(lb_ctx *ctx, const StepArgs &a, int K) {
+    const WavePick p = pick(ctx, K, a.rho_out != nullptr);
+    WaveArgs w;
+    w.row_off = a.trace_row ? ctx->row_off : nullptr;
+    w.rec_x = ctx->row_x;
+    w.rec_id = ctx->row_id;
+    w.rec_y = ctx->row_y;
+    w.outer = outer_weight(ctx, K);
+    strips_of(w, ctx->nx, K, a.sponge_w, ctx->cfg.boundary == LB_PERIODIC);
+    shape(w, ctx->ny, K, p.ctas);
+    cudaError_t e = cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "wavefront shared memory");
+    e = launch_pdl(p.fn, dim3((w.tasks + kWarpsPerCta - 1) / kWarpsPerCta), dim3(kCtaThreads), p.smem,
+                   ctx->stream, a, w);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "wavefront launch");
+    return LB_OK;
+}
+
+// ---------------------------------------------------------------- fused launches --
+// cfg.time_block values (wave_launch_args takes them in launches of 2, 4 or 6 steps)
+bool tb_supported(int Q, int K) {
+    return Q == 5 ? K == 2 || K == 4 || K == 6 || K == 8 || K == 16 : K == 2 || K == 4;
+}
+
+// K fused steps of the context from a non-raw state; the caller keeps them inside the trace
+// buffer and the rho tape.
+lb_status tb_launch(lb_ctx *ctx, int K) {
+    StepArgs a = base_args(ctx);
+    a.in = ctx->pop[ctx->cur];
+    a.out = ctx->pop[ctx->cur ^ 1];
+    a.t = ctx->t;
+    a.raw = 0;
+    const long long row = ctx->t - ctx->t_rec0;
+    a.trace_row = (ctx->trace && ctx->row_off && row >= 0 && row + K <= ctx->trace_cap)
+                      ? ctx->trace + row * ctx->nrec : nullptr;
+    a.rho_out = tape_row(ctx, ctx->t);  // level j at rho_out + j plane
+    a.rho_stride = (long long)ctx->ny * ctx->pitch;
+    lb_status st = ctx->cfg.storage == LB_BF16 && ctx->cfg.time_block > 1
+                       ? tb5_launch_args(ctx, a, K)
+                       : wave_launch_args(ctx, a, K);
+    if (st != LB_OK) return st;
+    ctx->cur ^= 1;
+    ctx->t += K;
+    return LB_OK;
+}
+
+// ------------------------------------------------------------- served batches --
+// One launch of wave_batch_kernel: the descriptors of its n shots in one staging block,
+// [n] StepArgs, [n] WaveArgs, [n + 1] block prefixes.
+namespace {
+size_t up256(size_t v) { return (v + 255) / 256 * 256; }
+struct BatchLayout {
+    StepArgs *a;
+    WaveArgs *w;
+    int *first;
+};
+BatchLayout batch_layout(void *base, int n) {
+    char *p = static_cast<char *>(base);
+    BatchLayout L;
+    L.a = reinterpret_cast<StepArgs *>(p);
+    p += up256(n * sizeof(StepArgs));
+    L.w = reinterpret_cast<WaveArgs *>(p);
+    p += up256(n * sizeof(WaveArgs));
+    L.first = reinterpret_cast<int *>(p);
+    return L;
+}
+// tasks and shape of one shot at about H rows per chunk
+int batch_shape(const lb_ctx *c, int H, WaveArgs &w) {
+    w.outer = outer_weight(c, kServeSteps);
+    strips_of(w, c->nx, kServeSteps, c->cfg.sponge_width, c->cfg.boundary == LB_PERIODIC);
+    H = std::max(1, std::min(c->ny, H));
+    return (int)set_chunks(w, c->ny, (c->ny + H - 1) / H);
+}
+int ctas_of(int tasks) { return (tasks + kWarpsPerCta - 1) / kWarpsPerCta; }
+}  // namespace
+
+size_t wave_batch_bytes(int n) {
+    return up256(n * sizeof(StepArgs)) + up256(n * sizeof(WaveArgs)) + up256((n + 1) * sizeof(int));
+}
+
+bool wave_batch_ready(const lb_ctx *ctx) {
+    constexpr int K = kServeSteps;
+    if (ctx->Q != 5 || !wave_supported(ctx) || ctx->raw || ctx->ckpt_every > 0) return false;
+    if (ctx->rho_tape) {  // BF16 batches keep FP32 between the steps; a tape wants every step's BF16
+        const long long row = ctx->t - ctx->tape_t0;
+        if (ctx->cfg.storage != LB_F32 || row < 0 || row + K > ctx->tape_cap) return false;
+    }
+    if (ctx->nrec > 0) {
+        const long long row = ctx->t - ctx->t_rec0;
+        if (!ctx->row_off || row < 0 || row + K > ctx->trace_cap) return false;
+    }
+    return true;
+}
+
+int wave_batch_rows(lb_ctx *const *ctxs, int n) {
+    // the rows per warp of shape(), over all shots' strips
+    long long rows = 0;
+    int ny = 1;
+    for (int k = 0; k < n; k++) {
+        WaveArgs w;
+        strips_of(w, ctxs[k]->nx, kServeSteps, ctxs[k]->cfg.sponge_width, false);
+        rows += (long long)w.strips * ctxs[k]->ny;
+        ny = std::max(ny, ctxs[k]->ny);
+    }
+    const long long slots1 = (long long)sm_count() * kWarpsPerCta;
+    long long cost = -1, best = 1;
+    for (int m = 1; m <= 4; m++) {
+        const long long H = std::min<long long>(ny, (rows + m * slots1 - 1) / (m * slots1));
+        const long long c = (H + 2 * kServeSteps) * (4 + m);
+        if (cost < 0 || c < cost) cost = c, best = H;
+    }
+    return (int)best;
+}
+
+bool wave_batch_round(lb_ctx *const *ctxs, int n) {
+    static std::atomic<int> l2{-1};
+    int bytes = l2.load(std::memory_order_relaxed);
+    if (bytes < 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&bytes, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
+            cudaGetLastError();
+            bytes = 0;
+        }
+        l2.store(bytes, std::memory_order_relaxed);
+    }
+    long long rows = 0, state = 0;
+    for (int k = 0; k < n; k++) {
+        rows += (long long)((ctxs[k]->nx + 247) / 248) * ctxs[k]->ny;
+        state += 2LL * ctxs[k]->Q * ctxs[k]->ny * ctxs[k]->pitch * ctxs[k]->ebytes;
+    }
+    return !(rows > 11LL * 3 * sm_count() && 4 * state > 3LL * bytes);
+}
+
+int wave_batch_blocks(const lb_ctx *ctx, int H) {
+    WaveArgs w;
+    return ctas_of(batch_shape(ctx, H, w));
+}
+
+// Fill the host staging block `h` for kServeSteps steps of ctxs[0 .. n), about H output rows per
+// warp (advancing their time and buffers as if the launch ran); returns the block count.
+int wave_batch_fill(lb_ctx *const *ctxs, int n, int H, void *h) {
+    BatchLayout L = batch_layout(h, n);
+    int blocks = 0;
+    for (int k = 0; k < n; k++) {
+        lb_ctx *ctx = ctxs[k];
+        StepArgs a = base_args(ctx);
+        a.in = ctx->pop[ctx->cur];
+        a.out = ctx->pop[ctx->cur ^ 1];
+        a.t = ctx->t;
+        a.raw = 0;
+        a.rho_out = tape_row(ctx, ctx->t);
+        a.rho_stride = (long long)ctx->ny * ctx->pitch;
+        const long long row = ctx->t - ctx->t_rec0;
+        a.trace_row = ctx->nrec > 0 ? ctx->trace + row * ctx->nrec : nullptr;
+        WaveArgs w;
+        w.row_off = a.trace_row ? ctx->row_off : nullptr;
+        w.rec_x = ctx->row_x;
+        w.rec_id = ctx->row_id;
+        w.rec_y = ctx->row_y;
+    w.rec_y = ctx->row_y;
+        const int tasks = batch_shape(ctx, H, w);
+        L.a[k] = a;
+        L.w[k] = w;
+        L.first[k] = blocks;
+        blocks += ctas_of(tasks);
+        ctx->cur ^= 1;
+        ctx->t += kServeSteps;
+    }
+    L.first[n] = blocks;
+    return blocks;
+}
+
+cudaError_t wave_batch_launch(const void *d, int n, int blocks, bool mrt, int storage, bool round,
+                              cudaStream_t stream) {
+    if (n < 1 || blocks < 1) return cudaErrorInvalidValue;
+    const WaveBatchPick p = storage == LB_BF16 ? pick_batch_bf16(mrt, round) : pick_batch_f32(mrt);
+    cudaError_t e = cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+    if (e != cudaSuccess) return e;
+    BatchLayout L = batch_layout(const_cast<void *>(d), n);
+    return launch_pdl(p.fn, dim3(blocks), dim3(kCtaThreads), p.smem, stream, (const StepArgs *)L.a,
+                      (const WaveArgs *)L.w, (const int *)L.first, n);
+}

@@ -1,0 +1,75 @@
+"""Several steps per launch (csrc/wave.cuh) against one launch per step, bit for bit.
+
+The fused launch does a site's arithmetic operation by operation as the one-step kernels do and
+rounds 16-bit storage at every step, so states and traces are equal, not merely close.  The
+shapes are the places where it can go wrong: grids narrower than a strip, strips that end one
+column past the last, odd widths at a periodic seam, sponges that cover a strip, chunks tall
+enough for the path without checks, receivers on every kind of row and in dense rows, a source
+in a recomputed column, and step counts that leave every remainder.
+"""
+import numpy as np
+import pytest
+
+from paper_1704_03172_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sim_cls():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1704_03172_gb300 import build
+    build.build()
+    from paper_1704_03172_gb300.sim import LBSim
+    return LBSim
+
+
+def _equal(sim_cls, Q, coll, tau, storage, boundary, nx, ny, sponge, medium, steps, time_block):
+    import torch
+    rng = np.random.default_rng(nx * 7 + ny)
+    if medium == "random":
+        c = W.random_medium(nx, ny, 5, 0.5, 1.0)
+    else:
+        c = np.where(np.arange(ny)[:, None] > ny // 2, 1.0, 0.6) * np.ones((ny, nx))
+    g0 = torch.tensor(rng.normal(size=(Q, ny, nx)).astype(np.float32), device="cuda")
+    rec = [np.stack([rng.integers(0, nx, 11), rng.integers(0, ny, 11)], 1)]
+    if nx >= 64:  # a sparse and a dense line (more than 32 receivers in a strip)
+        rec += [W.line_receivers(nx // 9, ny // 4, 0, nx), W.line_receivers(nx, ny // 3, 0, nx)]
+    rec = np.concatenate(rec).astype(np.int32)
+    wav, out = rng.normal(size=steps - 4), []
+    for how in (dict(step_kernel="direct"), dict(time_block=time_block)):
+        sim = sim_cls(c.astype(np.float32), lattice=Q, collision=coll, tau=tau,
+                      s=W.mrt_rates(Q, W.DEFAULT_SEED + 2), storage=storage, boundary=boundary,
+                      sponge_width=sponge, c_ref=1.0, w_ref=(0.0, 0.01, 0.24), **how)
+        sim.set_source(nx // 3, ny // 2, wav)
+        sim.set_receivers(rec, steps)
+        sim.set_state(g0)
+        sim.step(steps)
+        out.append((sim.state().clone(), sim.traces(steps).clone()))
+        sim.close()
+    assert torch.equal(out[0][0], out[1][0])
+    assert torch.equal(out[0][1], out[1][1])
+
+
+SMALL = [(3, 5), (5, 300), (57, 31), (64, 40), (112, 33), (121, 7), (257, 131)]
+
+
+@pytest.mark.parametrize("Q,coll,tau", [(5, "bgk", 0.5), (5, "bgk", 0.8), (5, "mrt", 0.5),
+                                        (9, "bgk", 0.8), (9, "mrt", 0.5)])
+@pytest.mark.parametrize("boundary", ["zero", "periodic"])
+def test_small_grids(sim_cls, Q, coll, tau, boundary):
+    for nx, ny in SMALL:
+        for sponge, medium in ((0, "layers"), (6, "random")):
+            _equal(sim_cls, Q, coll, tau, "f32", boundary, nx, ny, sponge, medium, 23, 4)
+
+
+@pytest.mark.parametrize("Q,coll,tau", [(5, "bgk", 0.5), (5, "bgk", 0.8), (5, "mrt", 0.5),
+                                        (9, "bgk", 0.8), (9, "mrt", 0.5)])
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+def test_large_grids_fuse_unasked(sim_cls, Q, coll, tau, storage):
+    for boundary, nx, ny, sponge, medium in (("zero", 2000, 1500, 40, "layers"),
+                                             ("periodic", 2501, 1333, 0, "random"),
+                                             ("zero", 3900, 2100, 40, "random")):
+        _equal(sim_cls, Q, coll, tau, storage, boundary, nx, ny, sponge, medium, 23, 1)
