@@ -648,13 +648,14 @@ extern "C" lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *g
     // last one goes to `last` (when given); rho(t) goes to tape[t - from] (when given).
     // Several steps per launch where the fused kernel has them (not from a raw state): its
     // results are the one-step kernels', so a BF16 replay reproduces the forward run.
-    const bool fuse = wave_supported(ctx) && wave_pays(ctx);
+    const bool fuse = wave_supported(ctx);
     lb_status rst = LB_OK;
     auto replay = [&](const void *in, bool raw, long long from, int n, void *last, bool record) {
         int x = 0;
         for (int m = 0; m < n;) {
             const bool first_raw = raw && m == 0;
-            const int len = fuse && !first_raw ? wave_steps(ctx, n - m) : 1;
+            const Fuse f = fuse && !first_raw ? fuse_steps(ctx, n - m) : Fuse{1, false};
+            const int len = f.steps;
             StepArgs a = base;
             a.in = in;
             a.out = (m + len == n && last) ? last : X[x];
@@ -663,7 +664,7 @@ extern "C" lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *g
             a.rho_out = record ? tape + (size_t)m * plane : nullptr;
             a.rho_stride = (long long)plane;
             if (len > 1) {
-                if (rst == LB_OK) rst = wave_launch_args(ctx, a, len);
+                if (rst == LB_OK) rst = fuse_launch_args(ctx, a, f);
             } else if (ctx->staged) {
                 stream_launch(ctx, a, 0);  // cannot fail once the forward run has stepped
             } else {

@@ -150,6 +150,10 @@ void ckpt_reset(lb_ctx *ctx);
 void tape_reset(lb_ctx *ctx);
 float *tape_row(const lb_ctx *ctx, long long t);
 
+struct Fuse {
+    int steps;  // of the next launch (1: the one-step kernels)
+    bool tile;  // on register tiles (tile.cuh)
+};
 // several steps per launch (wave.cu): the cfg.time_block values, and K steps of a context
 bool tb_supported(int Q, int K);
 // TMA-staged persistent step (stream_step.cu): one LB step of the context's grid
@@ -158,7 +162,7 @@ lb_status stream_launch(lb_ctx *ctx, const lbk::StepArgs &a, int rec_blocks);
 // from the per-row lists of wave_set_receivers (rec_off nullptr: none this step)
 lb_status stream_launch_aa(lb_ctx *ctx, const lbk::StepArgs &a, bool exchange, const int *rec_off,
                            const int *rec_x, const int *rec_id);
-lb_status tb_launch(lb_ctx *ctx, int K);
+lb_status tb_launch(lb_ctx *ctx, Fuse f);
 // in-place streaming (aa.cu): n steps of an LB_STREAM_AA context
 lb_status aa_step(lb_ctx *ctx, int n);
 // warp wavefront (wave.cu): 2, 4 or 6 steps of a D2Q5, 2 or 4 of a D2Q9 grid per launch, FP32 or
@@ -166,10 +170,9 @@ lb_status aa_step(lb_ctx *ctx, int n);
 // it pays without being asked for, the steps the next launch takes of n wanted, the receivers' row
 // lists, and the launch
 bool wave_supported(const lb_ctx *ctx);
-bool wave_pays(const lb_ctx *ctx);
-int wave_steps(const lb_ctx *ctx, int n);
+Fuse fuse_steps(const lb_ctx *ctx, int n);
 lb_status wave_set_receivers(lb_ctx *ctx, const int *xy, int nrec);
-lb_status wave_launch_args(lb_ctx *ctx, const lbk::StepArgs &a, int K);
+lb_status fuse_launch_args(lb_ctx *ctx, const lbk::StepArgs &a, Fuse f);
 // its served batches of D2Q5 shots, kServeSteps steps per launch: staging bytes of one launch's
 // descriptors, whether a shot can take the steps now, the rows per warp that suit n shots
 // together, a shot's CTAs at H rows per warp, the fill (advancing the shots) and the launch from

@@ -1033,9 +1033,10 @@ lb_status lb_step(lb_ctx *ctx, int n) {
 // Steps of the next launch, of which `left` are wanted: several where a fused kernel takes
 // them, never across a checkpoint time, the end of the trace buffer or of the rho tape (single
 // steps keep all three exact), and one from a raw state.
-static int fused_steps(const lb_ctx *ctx, int left) {
+static Fuse next_launch(const lb_ctx *ctx, int left) {
     const int T = ctx->cfg.time_block;
-    if (ctx->raw || left < 2) return 1;
+    const Fuse one{1, false};
+    if (ctx->raw || left < 2) return one;
     long long room = left;
     if (ctx->ckpt_every > 0)
         room = std::min<long long>(room, ctx->ckpt_every - (ctx->t - ctx->ckpt_t0) % ctx->ckpt_every);
@@ -1045,10 +1046,10 @@ static int fused_steps(const lb_ctx *ctx, int left) {
     const bool taping = ctx->rho_tape && trow < ctx->tape_cap;
     if (taping) room = std::min<long long>(room, ctx->tape_cap - trow);
     if (T > 1 && ctx->cfg.storage == LB_BF16)  // FP32 between the levels: no rho record
-        return room >= T && !taping ? T : 1;
-    if (T > 1) return wave_steps(ctx, (int)std::min<long long>(room, T));
-    if (ctx->cfg.step_kernel != LB_STEP_AUTO || !wave_supported(ctx) || !wave_pays(ctx)) return 1;
-    return wave_steps(ctx, (int)std::min<long long>(room, 1 << 20));
+        return room >= T && !taping ? Fuse{T, false} : one;
+    if (T > 1) return fuse_steps(ctx, (int)std::min<long long>(room, T));
+    if (ctx->cfg.step_kernel != LB_STEP_AUTO || !wave_supported(ctx)) return one;
+    return fuse_steps(ctx, (int)std::min<long long>(room, 1 << 20));
 }
 
 static lb_status step_n(lb_ctx *ctx, int n) {
@@ -1065,10 +1066,10 @@ static lb_status step_n(lb_ctx *ctx, int n) {
             lb_status st = ckpt_maybe_save(ctx);
             if (st != LB_OK) return st;
         }
-        const int K = fused_steps(ctx, n - k);
-        lb_status st = K > 1 ? tb_launch(ctx, K) : launch_step(ctx, fn, a);
+        const Fuse f = next_launch(ctx, n - k);
+        lb_status st = f.steps > 1 ? tb_launch(ctx, f) : launch_step(ctx, fn, a);
         if (st != LB_OK) return st;
-        k += K;
+        k += f.steps;
     }
     return check_launch(ctx, "step_kernel");
 }

@@ -8,12 +8,14 @@
 
 #include "lb_kernels.cuh"
 #include "lb_runtime.h"
+#include "tile.cuh"
 #include "wave.cuh"
 #include "wave_host.h"
 
 using namespace lbk;
 using namespace lbrt;
 using namespace lbwave;
+using namespace lbtile;
 
 namespace lbwave {
 WavePick pick_d2q5_f32(int ck, int K, bool rec) {
@@ -114,13 +116,13 @@ bool wave_supported(const lb_ctx *c) {
 
 // A launch of four steps takes about 10 us however small the grid is, and longer with receivers;
 // a step alone takes 3 (128^2: 3.5 us a step fused against 3.0; 512^2: 4.6 against 5.4).
-bool wave_pays(const lb_ctx *c) { return (long long)c->ny * c->pitch >= (128LL << 10); }
+static bool wave_pays(const lb_ctx *c) { return (long long)c->ny * c->pitch >= (128LL << 10); }
 
 // Six steps (three CTAs per SM) beat four (four CTAs) where HBM is the limit: FP32 BGK grids well
 // beyond L2 (8192^2: 645 GLUPS against 560, 3000 x 2500: 470 against 440; 2048^2, 168 MB: 379
 // against 388).  MRT and BF16 are bound by issue first and run four (4096^2 MRT: 525 against
 // 470, BF16: 541 against 493).
-int wave_steps(const lb_ctx *c, int n) {
+static int wave_steps(const lb_ctx *c, int n) {
     if (c->Q == 5 && c->cfg.storage == LB_F32 && c->cfg.collision == LB_BGK && n >= 6 && n != 8 &&
         2LL * 5 * 4 * c->ny * c->pitch >= (200LL << 20))
         return 6;
@@ -158,15 +160,8 @@ lb_status wave_set_receivers(lb_ctx *ctx, const int *xy, int nrec) {
     return LB_OK;
 }
 
-// K fused steps with the caller's arguments (a.in must not be raw); receivers when
-// a.trace_row is set and the row lists exist; rho of every level when a.rho_out is set.
-lb_status wave_launch_args(lb_ctx *ctx, const StepArgs &a, int K) {
+static lb_status wave_launch(lb_ctx *ctx, const StepArgs &a, WaveArgs w, int K) {
     const WavePick p = pick(ctx, K, a.rho_out != nullptr);
-    WaveArgs w;
-    w.row_off = a.trace_row ? ctx->row_off : nullptr;
-    w.rec_x = ctx->row_x;
-    w.rec_id = ctx->row_id;
-    w.rec_y = ctx->row_y;
     w.outer = outer_weight(ctx, K);
     strips_of(w, ctx->nx, K, a.sponge_w, ctx->cfg.boundary == LB_PERIODIC);
     shape(w, ctx->ny, K, p.ctas);
@@ -178,15 +173,85 @@ lb_status wave_launch_args(lb_ctx *ctx, const StepArgs &a, int K) {
     return LB_OK;
 }
 
+// tiles of K steps, and how many to a row of tiles
+static int tiles_of(const lb_ctx *c, int K, int *tx) {
+    const int ox = kSide - 2 * halo_x(K), oy = kSide - 2 * K;
+    *tx = (c->nx + ox - 1) / ox;
+    return *tx * ((c->ny + oy - 1) / oy);
+}
+
+static lb_status tile_launch(lb_ctx *ctx, const StepArgs &a, const WaveArgs &rec, int K) {
+    TileArgs t;
+    t.rec = rec;
+    t.K = K;
+    const int tiles = tiles_of(ctx, K, &t.tx), ctas = tiles <= sm_count() ? 1 : 2;
+    const int ck = collision_kind(ctx);
+    const bool rho = a.rho_out != nullptr;
+    const TileFn fn = ctx->cfg.storage == LB_BF16 ? pick_tile_bf16(ck, rho, ctas)
+                                                  : pick_tile_f32(ck, rho, ctas);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(Shared));
+    if (e == cudaSuccess)
+        e = launch_pdl(fn, dim3(tiles), dim3(kTileThreads), sizeof(Shared),
+                       ctx->stream, a, t);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "tile launch");
+    return LB_OK;
+}
+
+// f.steps fused steps with the caller's arguments (a.in must not be raw); receivers when
+// a.trace_row is set and the row lists exist; rho of every level when a.rho_out is set.
+lb_status fuse_launch_args(lb_ctx *ctx, const StepArgs &a, Fuse f) {
+    WaveArgs w = {};
+    w.row_off = a.trace_row ? ctx->row_off : nullptr;
+    w.rec_x = ctx->row_x;
+    w.rec_id = ctx->row_id;
+    w.rec_y = ctx->row_y;
+    w.per = ctx->cfg.boundary == LB_PERIODIC ? 1 : 0;
+    return f.tile ? tile_launch(ctx, a, w, f.steps) : wave_launch(ctx, a, w, f.steps);
+}
+
+// About what a launch of K steps on tiles takes, in 0.01 us, from GB300 times of 128^2 to 2048^2
+// grids for K = 4 .. 16: with q tiles per SM, 5.2 + 0.54 K us up to one, then the larger of
+// 6 + 1.35 K (two share an SM) and 4 + q (2.5 + 0.62 K).
+static long long tile_cost(const lb_ctx *c, int K) {
+    int tx;
+    const long long t = tiles_of(c, K, &tx), sms = sm_count();
+    if (t <= sms) return 520 + 54 * K;
+    return std::max<long long>(600 + 135 * K, 400 + t * (250 + 62 * K) / sms);
+}
+
+// The next launch of n wanted steps.  D2Q5 grids up to 3.5 million sites go on tiles, in launches
+// of the K <= 16 steps that cost least each (evened out over the launches that n takes), where
+// that beats single steps of about 3.1 us + 6 ps a site; above, and for D2Q9, the wavefront is
+// faster (2048^2: 10.8 against 11.0 us a step, 4096^2: 29 against 44).
+Fuse fuse_steps(const lb_ctx *c, int n) {
+    const long long sites = (long long)c->ny * c->pitch;
+    if (c->Q == 5 && sites < 3500000) {
+        if (n < 2) return Fuse{1, false};
+        int best = 2;
+        long long cost = -1;
+        for (int K = 2; K <= 16; K += 2) {
+            const long long x = tile_cost(c, K);
+            if (cost < 0 || x * best < cost * K) cost = x, best = K;
+        }
+        const int launches = (n + best - 1) / best, K = (n + launches - 1) / launches;
+        if (tile_cost(c, K) >= K * (310 + sites * 6 / 10000)) return Fuse{1, false};
+        return Fuse{K, true};
+    }
+    if (!wave_pays(c) && c->cfg.time_block <= 1) return Fuse{1, false};
+    return Fuse{wave_steps(c, n), false};
+}
+
 // ---------------------------------------------------------------- fused launches --
-// cfg.time_block values (wave_launch_args takes them in launches of 2, 4 or 6 steps)
+// cfg.time_block values (fuse_steps takes them in launches that suit)
 bool tb_supported(int Q, int K) {
     return Q == 5 ? K == 2 || K == 4 || K == 6 || K == 8 || K == 16 : K == 2 || K == 4;
 }
 
 // K fused steps of the context from a non-raw state; the caller keeps them inside the trace
 // buffer and the rho tape.
-lb_status tb_launch(lb_ctx *ctx, int K) {
+lb_status tb_launch(lb_ctx *ctx, Fuse f) {
+    const int K = f.steps;
     StepArgs a = base_args(ctx);
     a.in = ctx->pop[ctx->cur];
     a.out = ctx->pop[ctx->cur ^ 1];
@@ -199,7 +264,7 @@ lb_status tb_launch(lb_ctx *ctx, int K) {
     a.rho_stride = (long long)ctx->ny * ctx->pitch;
     lb_status st = ctx->cfg.storage == LB_BF16 && ctx->cfg.time_block > 1
                        ? tb5_launch_args(ctx, a, K)
-                       : wave_launch_args(ctx, a, K);
+                       : fuse_launch_args(ctx, a, f);
     if (st != LB_OK) return st;
     ctx->cur ^= 1;
     ctx->t += K;

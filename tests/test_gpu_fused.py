@@ -1,4 +1,4 @@
-"""Several steps per launch (csrc/wave.cuh) against one launch per step, bit for bit.
+"""Several steps per launch (csrc/wave.cuh, csrc/tile.cuh) against one launch per step, bit for bit.
 
 The fused launch does a site's arithmetic operation by operation as the one-step kernels do and
 rounds 16-bit storage at every step, so states and traces are equal, not merely close.  The
@@ -69,7 +69,22 @@ def test_small_grids(sim_cls, Q, coll, tau, boundary):
                                         (9, "bgk", 0.8), (9, "mrt", 0.5)])
 @pytest.mark.parametrize("storage", ["f32", "bf16"])
 def test_large_grids_fuse_unasked(sim_cls, Q, coll, tau, storage):
-    for boundary, nx, ny, sponge, medium in (("zero", 2000, 1500, 40, "layers"),
-                                             ("periodic", 2501, 1333, 0, "random"),
+    for boundary, nx, ny, sponge, medium in (("zero", 2700, 1500, 40, "layers"),
+                                             ("periodic", 2501, 1433, 0, "random"),
+                                             ("periodic", 57, 62000, 5, "layers"),
+                                             ("zero", 121, 31001, 6, "random"),
                                              ("zero", 3900, 2100, 40, "random")):
         _equal(sim_cls, Q, coll, tau, storage, boundary, nx, ny, sponge, medium, 23, 1)
+
+
+# D2Q5 grids up to 3.5 million sites run on register tiles: one tile, tiles that end one column
+# or row past the last, periodic grids smaller than a region, more than one tile per SM, and step
+# counts that give launches of 2 .. 16 steps, odd ones among them
+@pytest.mark.parametrize("coll,tau", [("bgk", 0.5), ("bgk", 0.8), ("mrt", 0.5)])
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("boundary", ["zero", "periodic"])
+def test_tiles(sim_cls, coll, tau, storage, boundary):
+    for nx, ny, steps in ((3, 5, 18), (33, 32, 34), (64, 64, 12), (65, 129, 50), (257, 131, 8),
+                          (512, 400, 31), (801, 700, 26), (1531, 1187, 15)):
+        for sponge, medium in ((0, "layers"), (9, "random")):
+            _equal(sim_cls, 5, coll, tau, storage, boundary, nx, ny, sponge, medium, steps, 1)
