@@ -134,17 +134,26 @@ struct StepArgs {
     float *trace_row;        // pressure row for time t, or null
     const int *rec_col;      // column of receiver r in the trace row (nullptr: r)
     // FP16 storage: per-population power-of-two scale, value = stored * scale.
-    // Three device slots rotate.  The scale of the input buffer and the one chosen
+    // kScaleSlots device slots rotate.  The scale of the input buffer and the one chosen
     // for the output buffer are ready before the launch; every block folds its
     // max |output| into max_out, and a one-block kernel after the step derives the
-    // scale the next step will write with (scale_next, from 8 max|out| + |S[t+1]|)
-    // and clears max_next for it.  All nullptr for FP32 and BF16 storage (BF16 has
-    // the exponent range of FP32 and needs no range scale).
+    // scale the next step will write with (scale_next, from 8 max|out| + |S[t+1]|), a guess of
+    // the one after (scale_guess), and clears their max slots.  All nullptr for FP32 and BF16
+    // storage (BF16 has the exponent range of FP32 and needs no range scale).
     const float *scale_in;    // [9]
     const float *scale_out;   // [9]
     unsigned *max_out;        // [9][kMaxCopies] float bits of max |value| written
     float *scale_next;        // [9]
     unsigned *max_next;       // [9][kMaxCopies]
+    float *scale_guess;       // [9]
+    unsigned *max_guess;      // [9][kMaxCopies]
+    // Launches of two steps (wave.cu; nullptr for one): scale_out and max_out are those of the
+    // first step's values, which stay on the chip and are rounded as if stored; the second
+    // step's are stored under scale_two, the guess.  redo: the same launch once more, which ends at
+    // once unless the flag says that the guess was not the scale that single steps would use.
+    float *scale_two;         // [9]
+    unsigned *max_two;        // [9][kMaxCopies]
+    const unsigned *redo;
     // Adjoint replays only: rho(x, t) of the pulled state g(t), [ny][pitch] FP32
     // (nullptr otherwise); a time-blocked launch writes step j of its K at
     // rho_out + j rho_stride.
@@ -212,6 +221,7 @@ template <> __device__ __forceinline__ double src_at<double>(const StepArgs &a) 
     return a.src64[a.t];
 }
 
+constexpr int kScaleSlots = 5;         // FP16: a launch of two steps reads or writes five
 constexpr int kMaxCopies = 8;          // spread of the per-block atomicMax targets
 constexpr float kStoredTarget = 8192.f; // 16-bit: |stored| <= 2^13 for the predicted bound
 
@@ -1028,21 +1038,45 @@ __global__ void __launch_bounds__(kThreads, Q == 5   ? (sizeof(ST) == 4 ? 5 : 4)
     }
 }
 
-// FP16, after each step (one block): the scale the next step writes with, from
-// this step's maxima (8 max|out| + |S[t+1]| at or below kStoredTarget), and a
-// cleared max slot for the next step.  Launched as a programmatic dependent of the
-// step (it waits for the step's grid before it reads the maxima), so its launch and
-// the next step's overlap the step's last blocks.
-static __global__ void scale_update_kernel(StepArgs a, int Q) {
+// FP16, after each launch of one or two steps (one block): the scale the next step writes with,
+// from the last step's maxima (8 max|out| + |S| at or below kStoredTarget), a guess of the scale
+// after that one from the same maxima (they seldom cross a power of two from step to step), and
+// cleared max slots for both.  After two steps first the scale that the second step's values should
+// have been stored with, now that the first step's maxima are known; `redo` tells the launch that
+// follows whether it was another.  (The values before storing do not depend on it, so the
+// maxima stand.)  Launched as a programmatic dependent of the step (it waits for the step's grid
+// before it reads the maxima), so its launch and the next step's overlap the step's last blocks.
+static __global__ void scale_update_kernel(StepArgs a, int Q, unsigned *redo) {
     pdl_trigger_and_wait();
     const int i = threadIdx.x;
+    auto top = [&](const unsigned *p) {
+        float m = 0.f;
+        for (int c = 0; c < kMaxCopies; c++) m = fmaxf(m, __uint_as_float(p[i * kMaxCopies + c]));
+        return m;
+    };
+    auto source = [&](long long t) { return a.src_tab && t < a.src_nt ? fabsf(a.src_tab[t]) : 0.f; };
+    float m = 0.f, s = 1.f;
+    long long t = a.t + 1;
+    bool other = false;
+    if (i < Q) {
+        m = top(a.max_out);
+        s = a.scale_out[i];
+        if (a.scale_two) {
+            s = next_scale(m, source(t++), s);
+            other = s != a.scale_two[i];
+            a.scale_two[i] = s;
+            m = top(a.max_two);
+        }
+    }
+    if (a.scale_two) {
+        const bool any = __any_sync(0xffffffffu, other);
+        if (i == 0) *redo = any ? 1u : 0u;
+    }
     if (i >= Q) return;
-    float m = 0.f;
-    for (int c = 0; c < kMaxCopies; c++) m = fmaxf(m, __uint_as_float(a.max_out[i * kMaxCopies + c]));
-    const long long tn = a.t + 1;
-    const float S = (a.src_tab && tn < a.src_nt) ? fabsf(a.src_tab[tn]) : 0.f;
-    a.scale_next[i] = next_scale(m, S, a.scale_out[i]);
-    for (int c = 0; c < kMaxCopies; c++) a.max_next[i * kMaxCopies + c] = 0u;
+    const float next = next_scale(m, source(t), s);
+    a.scale_next[i] = next;
+    a.scale_guess[i] = next_scale(m, source(t + 1), next);
+    for (int c = 0; c < kMaxCopies; c++) a.max_next[i * kMaxCopies + c] = a.max_guess[i * kMaxCopies + c] = 0u;
 }
 
 // ------------------------------------------------------------ batched step --

@@ -29,8 +29,9 @@ struct lb_ctx {
     int n_mid = 0;
     bool staged = false;            // steps run the TMA-staged persistent kernel
     unsigned *fault = nullptr;      // device flag: a bounded wait in a kernel gave up
-    float *lp_scale = nullptr;      // FP16 storage: [3][9] per-population scales (slots)
-    unsigned *lp_max = nullptr;     // FP16 storage: [3][9][kMaxCopies] max |value| + counter
+    float *lp_scale = nullptr;      // FP16 storage: [kScaleSlots][9] per-population scales
+    unsigned *lp_max = nullptr;     // FP16 storage: [kScaleSlots][9][kMaxCopies] max |value|, then
+                                    // the flag of launches of two steps
     int lp_slot = 0;                // slot describing the current buffer
     double *inv_scratch = nullptr;  // lb_invariants: [ny][4] row partials + [4] result
     int ckpt_every = 0;             // adjoint checkpoints: state copied every ckpt_every steps
@@ -58,6 +59,7 @@ struct lb_ctx {
     int trace_cap = 0;
     long long t_rec0 = 0;
     long long t = 0;
+    long long n_launch = 0;         // kernels launched by lb_step (lb_info)
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     bool refined = false;
@@ -120,6 +122,10 @@ StepFn pick_step(const lb_ctx *c);
 lbk::StepArgs prepare_step(lb_ctx *ctx);  // FP32 / BF16 storage (no scale slots)
 GetFn pick_get_for(int Q, bool periodic, int storage);
 lb_status check_launch(lb_ctx *ctx, const char *what);
+// FP16: the scale and max slots of the next launch of one or two steps
+void f16_slots(lb_ctx *ctx, lbk::StepArgs &a, int steps);
+lb_status f16_update(lb_ctx *ctx, const lbk::StepArgs &a);  // and the scales after it
+unsigned *f16_redo(const lb_ctx *ctx);
 int round_up(int v, int m);
 // scale pointers of the current buffer (nullptr for FP32 storage)
 const float *current_scale(const lb_ctx *ctx);

@@ -595,13 +595,13 @@ lb_status lb_create(const lb_config *cfg, lb_ctx **out) {
                  (cfg->step_kernel == LB_STEP_AUTO && (cfg->storage == LB_BF16 ||
                                                        cfg->storage == LB_F16) && cfg->nx >= 1024));
     if (cfg->storage == LB_F16) {  // FP16 range scales (BF16 has FP32's range and needs none)
-        c->lp_scale = static_cast<float *>(dev_alloc(c, 3 * 9 * sizeof(float)));
-        c->lp_max = static_cast<unsigned *>(dev_alloc(c, (3 * 9 * kMaxCopies + 1) * sizeof(unsigned)));
+        c->lp_scale = static_cast<float *>(dev_alloc(c, kScaleSlots * 9 * sizeof(float)));
+        c->lp_max = static_cast<unsigned *>(dev_alloc(c, (kScaleSlots * 9 * kMaxCopies + 1) * sizeof(unsigned)));
         if (!c->lp_scale || !c->lp_max) return bail(fail(c, LB_ENOMEM, "scale buffers"));
-        std::vector<float> ones(27, 1.f);
-        cudaMemcpyAsync(c->lp_scale, ones.data(), 27 * sizeof(float), cudaMemcpyHostToDevice,
+        std::vector<float> ones(kScaleSlots * 9, 1.f);
+        cudaMemcpyAsync(c->lp_scale, ones.data(), ones.size() * sizeof(float), cudaMemcpyHostToDevice,
                         c->stream);
-        cudaMemsetAsync(c->lp_max, 0, (3 * 9 * kMaxCopies + 1) * sizeof(unsigned), c->stream);
+        cudaMemsetAsync(c->lp_max, 0, (kScaleSlots * 9 * kMaxCopies + 1) * sizeof(unsigned), c->stream);
     }
     // medium: c_map -> eta^2 (Eq. 0th lattice weight), on the device
     const float *cmap_dev = cfg->c_map;
@@ -831,8 +831,8 @@ static lb_status set_state_common(lb_ctx *ctx, const float *src, int on_device, 
     if (ctx->lp_scale) {
         // FP16: the written state's scale from its own max (slot s0), and the scale
         // the first step will write with (slot s1), whose max slot starts cleared
-        const int s0 = ctx->lp_slot, s1 = (s0 + 1) % 3;
-        cudaMemsetAsync(ctx->lp_max, 0, (3 * 9 * kMaxCopies + 1) * sizeof(unsigned), ctx->stream);
+        const int s0 = ctx->lp_slot, s1 = (s0 + 1) % kScaleSlots;
+        cudaMemsetAsync(ctx->lp_max, 0, (kScaleSlots * 9 * kMaxCopies + 1) * sizeof(unsigned), ctx->stream);
         a.t = ctx->t;
         a.max_out = ctx->lp_max + s0 * 9 * kMaxCopies;
         a.scale_next = ctx->lp_scale + s0 * 9;
@@ -941,20 +941,38 @@ StepArgs prepare_step(lb_ctx *ctx) {
     return a;
 }
 
+void f16_slots(lb_ctx *ctx, StepArgs &a, int steps) {
+    auto scale = [&](int k) { return ctx->lp_scale + (ctx->lp_slot + k) % kScaleSlots * 9; };
+    auto top = [&](int k) { return ctx->lp_max + (ctx->lp_slot + k) % kScaleSlots * 9 * kMaxCopies; };
+    a.scale_in = scale(0);
+    a.scale_out = scale(1);
+    a.max_out = top(1);
+    a.scale_two = steps == 2 ? scale(2) : nullptr;
+    a.max_two = steps == 2 ? top(2) : nullptr;
+    a.scale_next = scale(steps + 1);
+    a.max_next = top(steps + 1);
+    a.scale_guess = scale(steps + 2);
+    a.max_guess = top(steps + 2);
+    a.redo = nullptr;
+    ctx->lp_slot = (ctx->lp_slot + steps) % kScaleSlots;
+}
+
+unsigned *f16_redo(const lb_ctx *ctx) { return ctx->lp_max + kScaleSlots * 9 * kMaxCopies; }
+
+lb_status f16_update(lb_ctx *ctx, const StepArgs &a) {
+    cudaError_t e = launch_pdl(scale_update_kernel, dim3(1), dim3(32), 0, ctx->stream, a, ctx->Q,
+                               f16_redo(ctx));
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "scale update launch");
+    ctx->n_launch++;
+    return LB_OK;
+}
+
 // One uniform-grid step: state h^{t-1} in pop[cur] -> h^t in pop[cur ^ 1].
 lb_status launch_step(lb_ctx *ctx, StepFn fn, StepArgs &a) {
     a.in = ctx->pop[ctx->cur];
     a.out = ctx->pop[ctx->cur ^ 1];
     a.t = ctx->t;
-    if (ctx->lp_scale) {
-        const int s0 = ctx->lp_slot, s1 = (s0 + 1) % 3, s2 = (s0 + 2) % 3;
-        a.scale_in = ctx->lp_scale + s0 * 9;
-        a.scale_out = ctx->lp_scale + s1 * 9;
-        a.max_out = ctx->lp_max + s1 * 9 * kMaxCopies;
-        a.scale_next = ctx->lp_scale + s2 * 9;
-        a.max_next = ctx->lp_max + s2 * 9 * kMaxCopies;
-        ctx->lp_slot = s1;
-    }
+    if (ctx->lp_scale) f16_slots(ctx, a, 1);
     a.raw = ctx->raw ? 1 : 0;
     ctx->raw = false;
     a.rho_out = tape_row(ctx, ctx->t);  // forward rho tape for lb_adjoint, if recording
@@ -972,8 +990,8 @@ lb_status launch_step(lb_ctx *ctx, StepFn fn, StepArgs &a) {
         if (e != cudaSuccess) return cuda_fail(ctx, e, "step launch");
     }
     if (ctx->lp_scale) {
-        cudaError_t e = launch_pdl(scale_update_kernel, dim3(1), dim3(32), 0, ctx->stream, a, ctx->Q);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "scale update launch");
+        lb_status st = f16_update(ctx, a);
+        if (st != LB_OK) return st;
     }
     ctx->cur ^= 1;
     ctx->t += 1;

@@ -29,20 +29,7 @@ WavePick pick_d2q5_f32(int ck, int K, bool rec) {
 WaveBatchPick pick_batch_f32(bool mrt) { return pick_batch<float, false>(mrt); }
 }  // namespace lbwave
 
-namespace {
-
-int collision_kind(const lb_ctx *c) {
-    if (c->cfg.collision == LB_MRT) return kMrt;
-    return c->Q == 5 && (float)(1.0 / c->cfg.tau) == 2.f ? kLossless : kBgk;
-}
-
-WavePick pick(const lb_ctx *c, int K, bool rec) {
-    const int ck = collision_kind(c);
-    if (c->Q == 9)
-        return c->cfg.storage == LB_BF16 ? pick_d2q9_bf16(ck, K, rec) : pick_d2q9_f32(ck, K, rec);
-    return c->cfg.storage == LB_BF16 ? pick_d2q5_bf16(ck, K, rec) : pick_d2q5_f32(ck, K, rec);
-}
-
+namespace lbrt {
 int sm_count() {
     static std::atomic<int> sms{0};
     int v = sms.load(std::memory_order_relaxed);
@@ -56,6 +43,23 @@ int sm_count() {
         sms.store(v, std::memory_order_relaxed);
     }
     return v;
+}
+
+}  // namespace lbrt
+
+namespace {
+
+int collision_kind(const lb_ctx *c) {
+    if (c->cfg.collision == LB_MRT) return kMrt;
+    return c->Q == 5 && (float)(1.0 / c->cfg.tau) == 2.f ? kLossless : kBgk;
+}
+
+WavePick pick(const lb_ctx *c, int K, bool rec) {
+    const int ck = collision_kind(c);
+    if (c->Q == 9)
+        return c->cfg.storage == LB_BF16 ? pick_d2q9_bf16(ck, K, rec) : pick_d2q9_f32(ck, K, rec);
+    if (c->cfg.storage == LB_F16) return pick_d2q5_f16(ck, rec);
+    return c->cfg.storage == LB_BF16 ? pick_d2q5_bf16(ck, K, rec) : pick_d2q5_f32(ck, K, rec);
 }
 
 // What a row in the sponge counts against kInner: an iteration with sponge factors issues half as
@@ -111,7 +115,8 @@ void shape(WaveArgs &w, int ny, int K, int max_m) {
 
 bool wave_supported(const lb_ctx *c) {
     return (c->Q == 5 || c->Q == 9) && c->nz <= 1 && !c->refined && !c->aa && !c->slab_nyg &&
-           (c->cfg.storage == LB_F32 || c->cfg.storage == LB_BF16);
+           (c->cfg.storage == LB_F32 || c->cfg.storage == LB_BF16 ||
+            (c->cfg.storage == LB_F16 && c->Q == 5));
 }
 
 // A launch of four steps takes about 10 us however small the grid is, and longer with receivers;
@@ -227,6 +232,10 @@ static long long tile_cost(const lb_ctx *c, int K) {
 Fuse fuse_steps(const lb_ctx *c, int n) {
     const long long sites = (long long)c->ny * c->pitch;
     if (c->Q == 5 && sites < 3500000) {
+    // FP16: two, since its range scales are guessed no further ahead (a launch, the scale update and
+    // a second launch that mostly ends at once; 3001 x 1777: 25.5 us a step against 35.9)
+    if (c->cfg.storage == LB_F16)
+        return Fuse{n >= 2 && wave_pays(c) ? 2 : 1, false};
         if (n < 2) return Fuse{1, false};
         int best = 2;
         long long cost = -1;
@@ -264,9 +273,15 @@ lb_status tb_launch(lb_ctx *ctx, Fuse f) {
     a.rho_stride = (long long)ctx->ny * ctx->pitch;
     lb_status st = ctx->cfg.storage == LB_BF16 && ctx->cfg.time_block > 1
                        ? tb5_launch_args(ctx, a, K)
+    if (ctx->lp_scale) f16_slots(ctx, a, K);
                        : fuse_launch_args(ctx, a, f);
     if (st != LB_OK) return st;
     ctx->cur ^= 1;
+    if (st == LB_OK && ctx->lp_scale && (st = f16_update(ctx, a)) == LB_OK) {
+        a.redo = f16_redo(ctx);  // once more, where the second step's scale was another
+        ctx->n_launch++;
+        st = fuse_launch_args(ctx, a, f);
+    }
     ctx->t += K;
     return LB_OK;
 }

@@ -156,6 +156,67 @@ template <> struct Two<__nv_bfloat16> {
 };
 
 // the values at x - 1 and x + 1 of a lane's columns
+template <> struct Two<__half> {
+    __device__ static __forceinline__ uint32_t pack(float2 a) {
+        const __half2 h = __floats2half2_rn(a.x, a.y);
+        return *reinterpret_cast<const uint32_t *>(&h);
+    }
+    __device__ static __forceinline__ float2 unpack(uint32_t u) {
+        return __half22float2(*reinterpret_cast<const __half2 *>(&u));
+    }
+    __device__ static __forceinline__ float2 lds(uint32_t at) { return unpack(lds1(at)); }
+    __device__ static __forceinline__ void store(__half *o, float2 v) {
+        *reinterpret_cast<uint32_t *>(o) = pack(v);
+    }
+    __device__ static __forceinline__ float2 round(float2 v) { return unpack(pack(v)); }
+};
+
+// FP16's range scales (StepArgs): of the input, of the first step's values and of the output, and
+// the largest values of both steps.  The other types have none.
+template <int Q, typename ST> struct Range {
+    __device__ __forceinline__ explicit Range(const StepArgs &) {}
+    __device__ __forceinline__ float2 input(int, float2 v) const { return v; }
+    __device__ __forceinline__ float2 between(int, float2 v, bool) { return Two<ST>::round(v); }
+    __device__ __forceinline__ float2 output(int, float2 v) { return v; }
+    __device__ __forceinline__ void fold(const StepArgs &, int, bool) const {}
+};
+template <int Q> struct Range<Q, __half> {
+    float in[Q], mid[Q], imid[Q], out[Q], top1[Q], top2[Q];
+    __device__ __forceinline__ explicit Range(const StepArgs &a) {
+#pragma unroll
+        for (int i = 0; i < Q; i++) {
+            in[i] = a.scale_in[i];
+            mid[i] = a.scale_out[i];
+            imid[i] = 1.f / mid[i];  // exact: powers of two
+            out[i] = 1.f / a.scale_two[i];
+            top1[i] = top2[i] = 0.f;
+        }
+    }
+    __device__ __forceinline__ float2 input(int i, float2 v) const { return mul(f2(in[i]), v); }
+    // row: one of the chunk's own (warp-uniform)
+    __device__ __forceinline__ float2 between(int i, float2 v, bool row) {
+        if (row) top1[i] = fmaxf(top1[i], fmaxf(fabsf(v.x), fabsf(v.y)));
+        return mul(f2(mid[i]), Two<__half>::round(mul(f2(imid[i]), v)));
+    }
+    __device__ __forceinline__ float2 output(int i, float2 v) {
+        top2[i] = fmaxf(top2[i], fmaxf(fabsf(v.x), fabsf(v.y)));
+        return mul(f2(out[i]), v);
+    }
+    // every lane of the warp; own: its columns are output columns
+    __device__ __forceinline__ void fold(const StepArgs &a, int lane, bool own) const {
+#pragma unroll
+        for (int i = 0; i < Q; i++) {  // non-negative floats order as their bits
+            const unsigned m1 = __reduce_max_sync(0xffffffffu, own ? __float_as_uint(top1[i]) : 0u);
+            const unsigned m2 = __reduce_max_sync(0xffffffffu, own ? __float_as_uint(top2[i]) : 0u);
+            const int at = i * kMaxCopies + blockIdx.x % kMaxCopies;
+            if (lane == 0) {
+                atomicMax(a.max_out + at, m1);
+                atomicMax(a.max_two + at, m2);
+            }
+        }
+    }
+};
+
 __device__ __forceinline__ float2 from_left(float2 h) {
     return make_float2(__shfl_up_sync(0xffffffffu, h.y, 1), h.x);
 }
@@ -475,15 +536,15 @@ template <typename ST> struct Rows {
 // hold the source or receivers.
 template <int Q, int CK, int K, bool REC, typename ST, bool ROUND, bool FAST, int P>
 __device__ __forceinline__ void iterate(const StepArgs &a, const WaveArgs &w, const Lane &T,
-                                        Levels<Q, K> &S, Rows<ST> &at, int r, int rend,
-                                        int next_end, int &slot, bool sp) {
+                                        Levels<Q, K> &S, Rows<ST> &at, Range<Q, ST> &range, int r,
+                                        int rend, int next_end, int &slot, bool sp) {
     constexpr int NR = med_rows(K);
     cp_wait<kRing - 2>();
     float2 n[Q];  // level l's newest row r - l
     {
         const uint32_t s = slot_at<Q, ST>(T, slot);
 #pragma unroll
-        for (int i = 0; i < Q; i++) n[i] = Two<ST>::lds(s + i * kCols * (int)sizeof(ST));
+        for (int i = 0; i < Q; i++) n[i] = range.input(i, Two<ST>::lds(s + i * kCols * (int)sizeof(ST)));
         float2 m;
         if (a.mid) {
             const uint32_t u = lds1(slot_med<Q, ST>(T, slot)) >> (8 * (T.gxw & 2));
@@ -572,7 +633,7 @@ __device__ __forceinline__ void iterate(const StepArgs &a, const WaveArgs &w, co
             for (int i = 0; i < Q; i++) g[i] = mul(g[i], f);
         }
 #pragma unroll
-        for (int i = 0; i < Q; i++) n[i] = ROUND && l + 1 < K ? Two<ST>::round(g[i]) : g[i];
+        for (int i = 0; i < Q; i++) n[i] = ROUND && l + 1 < K ? range.between(i, g[i], FAST || (y >= T.Y0 && y < T.Y1)) : g[i];
     }
     // level K holds row r - K: an output row from Y0 on
     static_assert(CK != kLossless || K % 2 == 0, "the last level's sign");
@@ -582,7 +643,7 @@ __device__ __forceinline__ void iterate(const StepArgs &a, const WaveArgs &w, co
             for (int i = 0; i < Q; i++) n[i].y = 0.f;
         }
 #pragma unroll
-        for (int i = 0; i < Q; i++) Two<ST>::store(at.out + i * a.plane, n[i]);
+        for (int i = 0; i < Q; i++) Two<ST>::store(at.out + i * a.plane, range.output(i, n[i]));
     }
     at.out += a.pitch;
 }
@@ -702,19 +763,21 @@ __device__ __forceinline__ void sweep(const StepArgs &a, const WaveArgs &w, int 
     const int next_end = __any_sync(0xffffffffu, T.split) ? 0 : min(a.ny, rend);
     int slot = 0;
 #pragma unroll 1
+    Range<Q, ST> range(a);
     for (int r = rbeg; r < rend; r += 2) {
         const int e = fast_end(r);
 #pragma unroll 1
         for (; r + 1 < e; r += 2) {
-            iterate<Q, CK, K, REC, ST, ROUND, true, 0>(a, w, T, S, at, r, rend, next_end, slot, false);
-            iterate<Q, CK, K, REC, ST, ROUND, true, 1>(a, w, T, S, at, r + 1, rend, next_end, slot, false);
+            iterate<Q, CK, K, REC, ST, ROUND, true, 0>(a, w, T, S, at, range, r, rend, next_end, slot, false);
+            iterate<Q, CK, K, REC, ST, ROUND, true, 1>(a, w, T, S, at, range, r + 1, rend, next_end, slot, false);
         }
         if (r >= rend) break;
-        iterate<Q, CK, K, REC, ST, ROUND, false, 0>(a, w, T, S, at, r, rend, next_end, slot, sp);
+        iterate<Q, CK, K, REC, ST, ROUND, false, 0>(a, w, T, S, at, range, r, rend, next_end, slot, sp);
         if (r + 1 >= rend) break;
-        iterate<Q, CK, K, REC, ST, ROUND, false, 1>(a, w, T, S, at, r + 1, rend, next_end, slot, sp);
+        iterate<Q, CK, K, REC, ST, ROUND, false, 1>(a, w, T, S, at, range, r + 1, rend, next_end, slot, sp);
     }
 }
+    range.fold(a, T.lane, T.own);
 
 // resident CTAs per SM the registers are cut for
 template <int Q, int K, typename ST> constexpr int min_ctas() { return Q == 9 ? (K > 2 ? (sizeof(ST) == 4 ? 2 : 3) : 3) : K > 4 ? 3 : 4; }
@@ -727,6 +790,8 @@ __global__ void __launch_bounds__(kCtaThreads, min_ctas<Q, K, ST>())
     // 256^2: 3.1 against 2.5).
     asm volatile("griddepcontrol.wait;" ::: "memory");
     extern __shared__ __align__(16) unsigned char smem[];
+    if constexpr (sizeof(ST) == 2 && K == 2)
+        if (a.redo && *a.redo == 0u) return;  // (grid-uniform; FP16 only)
     float *tab = reinterpret_cast<float *>(smem + kWarpsPerCta * warp_bytes<Q, K, ST>());
     const int wi = threadIdx.x >> 5;
     sweep<Q, CK, K, REC, ST, ROUND>(a, w, blockIdx.x * kWarpsPerCta + wi, smem + wi * warp_bytes<Q, K, ST>(), tab);

@@ -29,6 +29,7 @@ template <int Q, int K, typename ST, bool ROUND> WavePick pick_rec(int ck, bool 
 
 WavePick pick_d2q5_f32(int ck, int K, bool rec);   // wave.cu
 WavePick pick_d2q5_bf16(int ck, int K, bool rec);  // wave_bf16.cu: rounded at every level
+WavePick pick_d2q5_f16(int ck, bool rec);          // wave_f16.cu: two steps
 WavePick pick_d2q9_f32(int ck, int K, bool rec);   // wave9.cu
 WavePick pick_d2q9_bf16(int ck, int K, bool rec);  // wave9_bf16.cu
 
