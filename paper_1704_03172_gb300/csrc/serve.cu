@@ -392,13 +392,17 @@ void pass(lb_server *S) {
         }
     }
     batched.swap(rest);
+    // one launch for FP32 and BF16 shots; a rho tape wants the BF16 of every step
+    auto tb_key = [&](const Req *r) {
+        return std::pair<bool, bool>(r->cfg.collision == LB_MRT,
+                                     round || (r->cfg.storage == LB_BF16 && r->ctx->rho_tape));
+    };
     std::stable_sort(tbs.begin(), tbs.end(),
-                     [&](const Req *a, const Req *b) { return key(a) < key(b); });
+                     [&](const Req *a, const Req *b) { return tb_key(a) < tb_key(b); });
     struct TbLaunch {
         size_t off;
         int n, blocks;
-        bool mrt;
-        int storage;
+        bool mrt, round;
         size_t g0, g1;
     };
     std::vector<TbLaunch> tb_launches;
@@ -406,7 +410,7 @@ void pass(lb_server *S) {
     if (!tbs.empty()) {
         for (size_t g0 = 0; g0 < tbs.size();) {  // staging bytes of every launch
             size_t g1 = g0;
-            while (g1 < tbs.size() && key(tbs[g1]) == key(tbs[g0])) g1++;
+            while (g1 < tbs.size() && tb_key(tbs[g1]) == tb_key(tbs[g0])) g1++;
             tb_bytes += nblk * wave_batch_bytes((int)(g1 - g0));
             g0 = g1;
         }
@@ -420,14 +424,14 @@ void pass(lb_server *S) {
         for (int j = 0; j < nblk && !tbs.empty(); j++) {
             for (size_t g0 = 0; g0 < tbs.size();) {
                 size_t g1 = g0;
-                while (g1 < tbs.size() && key(tbs[g1]) == key(tbs[g0])) g1++;
+                while (g1 < tbs.size() && tb_key(tbs[g1]) == tb_key(tbs[g0])) g1++;
                 cs.clear();
                 for (size_t q = g0; q < g1; q++) cs.push_back(tbs[q]->ctx);
                 const int n = (int)(g1 - g0);
                 const int blocks =
                     wave_batch_fill(cs.data(), n, tb_rows, static_cast<char *>(S->h_tb) + off);
-                const lb_config &c0 = tbs[g0]->cfg;
-                tb_launches.push_back({off, n, blocks, c0.collision == LB_MRT, c0.storage, g0, g1});
+                const auto [mrt, rounds] = tb_key(tbs[g0]);
+                tb_launches.push_back({off, n, blocks, mrt, rounds, g0, g1});
                 off += wave_batch_bytes(n);
                 g0 = g1;
             }
@@ -509,8 +513,8 @@ void pass(lb_server *S) {
         return;
     }
     for (const TbLaunch &L : tb_launches) {  // time-blocked blocks of K steps
-        e = wave_batch_launch(static_cast<char *>(S->d_tb) + L.off, L.n, L.blocks, L.mrt, L.storage,
-                              round, S->stream);
+        e = wave_batch_launch(static_cast<char *>(S->d_tb) + L.off, L.n, L.blocks, L.mrt, L.round,
+                              S->stream);
         if (e != cudaSuccess) {
             const std::string msg = std::string("time-blocked batch: ") + cudaGetErrorString(e);
             set_err(S, msg);

@@ -26,7 +26,7 @@ WavePick pick_d2q5_f32(int ck, int K, bool rec) {
                                      : pick_one<5, kBgk, 6, false, float, false>();
     return K == 4 ? pick_rec<5, 4, float, false>(ck, rec) : pick_rec<5, 2, float, false>(ck, rec);
 }
-WaveBatchPick pick_batch_f32(bool mrt) { return pick_batch<float, false>(mrt); }
+WaveBatchFn pick_batch_fp32(bool mrt) { return pick_batch<false>(mrt); }
 }  // namespace lbwave
 
 namespace lbrt {
@@ -322,10 +322,10 @@ size_t wave_batch_bytes(int n) {
 
 bool wave_batch_ready(const lb_ctx *ctx) {
     constexpr int K = kServeSteps;
-    if (ctx->Q != 5 || !wave_supported(ctx) || ctx->raw || ctx->ckpt_every > 0) return false;
-    if (ctx->rho_tape) {  // BF16 batches keep FP32 between the steps; a tape wants every step's BF16
+    if (ctx->Q != 5 || ctx->cfg.storage == LB_F16 || !wave_supported(ctx) || ctx->raw || ctx->ckpt_every > 0) return false;
+    if (ctx->rho_tape) {
         const long long row = ctx->t - ctx->tape_t0;
-        if (ctx->cfg.storage != LB_F32 || row < 0 || row + K > ctx->tape_cap) return false;
+        if (row < 0 || row + K > ctx->tape_cap) return false;
     }
     if (ctx->nrec > 0) {
         const long long row = ctx->t - ctx->t_rec0;
@@ -400,7 +400,7 @@ int wave_batch_fill(lb_ctx *const *ctxs, int n, int H, void *h) {
         w.rec_x = ctx->row_x;
         w.rec_id = ctx->row_id;
         w.rec_y = ctx->row_y;
-    w.rec_y = ctx->row_y;
+        w.bf16 = ctx->cfg.storage == LB_BF16 ? 1 : 0;
         const int tasks = batch_shape(ctx, H, w);
         L.a[k] = a;
         L.w[k] = w;
@@ -413,13 +413,15 @@ int wave_batch_fill(lb_ctx *const *ctxs, int n, int H, void *h) {
     return blocks;
 }
 
-cudaError_t wave_batch_launch(const void *d, int n, int blocks, bool mrt, int storage, bool round,
+cudaError_t wave_batch_launch(const void *d, int n, int blocks, bool mrt, bool round,
                               cudaStream_t stream) {
     if (n < 1 || blocks < 1) return cudaErrorInvalidValue;
-    const WaveBatchPick p = storage == LB_BF16 ? pick_batch_bf16(mrt, round) : pick_batch_f32(mrt);
-    cudaError_t e = cudaFuncSetAttribute(p.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
+    const WaveBatchFn fn = round ? pick_batch_round(mrt) : pick_batch_fp32(mrt);
+    constexpr int smem = cta_bytes<5, kServeSteps, float>();
+    static_assert(smem >= cta_bytes<5, kServeSteps, __nv_bfloat16>(), "room for either storage");
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     BatchLayout L = batch_layout(const_cast<void *>(d), n);
-    return launch_pdl(p.fn, dim3(blocks), dim3(kCtaThreads), p.smem, stream, (const StepArgs *)L.a,
+    return launch_pdl(fn, dim3(blocks), dim3(kCtaThreads), smem, stream, (const StepArgs *)L.a,
                       (const WaveArgs *)L.w, (const int *)L.first, n);
 }

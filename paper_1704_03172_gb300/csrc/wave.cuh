@@ -74,6 +74,7 @@ struct WaveArgs {
     int outer;           // what a row in the sponge counts (chunk_row)
     int tasks;           // warps with work
     int per;             // periodic boundary
+    int bf16;            // served batches: the shot's storage is BF16 (else FP32)
 };
 
 // First row of chunk k of n.  Rows in the sponge count `outer` and the others kInner, as their
@@ -797,10 +798,29 @@ __global__ void __launch_bounds__(kCtaThreads, min_ctas<Q, K, ST>())
     sweep<Q, CK, K, REC, ST, ROUND>(a, w, blockIdx.x * kWarpsPerCta + wi, smem + wi * warp_bytes<Q, K, ST>(), tab);
 }
 
-// Several independent D2Q5 grids ("shots") advanced by K steps in one launch: shot k owns blocks
-// [first[k], first[k + 1]) and reads its own descriptors (the served batches).
 template <bool MRT, int K, typename ST, bool ROUND>
-__global__ void __launch_bounds__(kCtaThreads, min_ctas<5, K, ST>())
+__device__ __forceinline__ void sweep_shot(const StepArgs &a, const WaveArgs &w, int block,
+                                           unsigned char *smem) {
+    float *tab = reinterpret_cast<float *>(smem + kWarpsPerCta * warp_bytes<5, K, ST>());
+    const int wi = threadIdx.x >> 5, task = block * kWarpsPerCta + wi;
+    unsigned char *mine = smem + wi * warp_bytes<5, K, ST>();
+    if constexpr (MRT) {
+        sweep<5, kMrt, K, true, ST, ROUND>(a, w, task, mine, tab);
+    } else {  // (block-uniform)
+        if (a.omega == 2.f)
+            sweep<5, kLossless, K, true, ST, ROUND>(a, w, task, mine, tab);
+        else
+            sweep<5, kBgk, K, true, ST, ROUND>(a, w, task, mine, tab);
+    }
+}
+
+// Several independent D2Q5 grids ("shots") advanced by K steps in one launch: shot k owns blocks
+// [first[k], first[k + 1]) and reads its own descriptors (the served batches).  FP32 and BF16 shots
+// share the launch (ROUND: the BF16 ones round at every step): a few small shots leave most of
+// the chip idle, and a launch of K steps takes its 10 us
+// however few they are (24 shots of 256^2 to 1024^2, 400 steps: 41 ms against 47 apart).
+template <bool MRT, int K, bool ROUND>
+__global__ void __launch_bounds__(kCtaThreads, min_ctas<5, K, float>())
     wave_batch_kernel(const StepArgs *__restrict__ args, const WaveArgs *__restrict__ waves,
                       const int *__restrict__ first, int nshots) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -822,17 +842,10 @@ __global__ void __launch_bounds__(kCtaThreads, min_ctas<5, K, ST>())
         s_blk = (int)blockIdx.x - first[lo];
     }
     __syncthreads();
-    float *tab = reinterpret_cast<float *>(smem + kWarpsPerCta * warp_bytes<5, K, ST>());
-    const int wi = threadIdx.x >> 5, task = s_blk * kWarpsPerCta + wi;
-    unsigned char *mine = smem + wi * warp_bytes<5, K, ST>();
-    if constexpr (MRT) {
-        sweep<5, kMrt, K, true, ST, ROUND>(sa, sw, task, mine, tab);
-    } else {  // (block-uniform)
-        if (sa.omega == 2.f)
-            sweep<5, kLossless, K, true, ST, ROUND>(sa, sw, task, mine, tab);
-        else
-            sweep<5, kBgk, K, true, ST, ROUND>(sa, sw, task, mine, tab);
-    }
+    if (sw.bf16)  // (block-uniform)
+        sweep_shot<MRT, K, __nv_bfloat16, ROUND>(sa, sw, s_blk, smem);
+    else
+        sweep_shot<MRT, K, float, false>(sa, sw, s_blk, smem);
 }
 
 using WaveFn = void (*)(const StepArgs, const WaveArgs);

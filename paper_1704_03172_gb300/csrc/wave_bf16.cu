@@ -6,7 +6,5 @@ WavePick pick_d2q5_bf16(int ck, int K, bool rec) {
     return K == 4 ? pick_rec<5, 4, __nv_bfloat16, true>(ck, rec)
                   : pick_rec<5, 2, __nv_bfloat16, true>(ck, rec);
 }
-WaveBatchPick pick_batch_bf16(bool mrt, bool round) {
-    return round ? pick_batch<__nv_bfloat16, true>(mrt) : pick_batch<__nv_bfloat16, false>(mrt);
-}
+WaveBatchFn pick_batch_round(bool mrt) { return pick_batch<true>(mrt); }
 }  // namespace lbwave

@@ -33,16 +33,11 @@ WavePick pick_d2q5_f16(int ck, bool rec);          // wave_f16.cu: two steps
 WavePick pick_d2q9_f32(int ck, int K, bool rec);   // wave9.cu
 WavePick pick_d2q9_bf16(int ck, int K, bool rec);  // wave9_bf16.cu
 
-struct WaveBatchPick {
-    WaveBatchFn fn;
-    int smem;
-};
-template <typename ST, bool ROUND> WaveBatchPick pick_batch(bool mrt) {
-    return {mrt ? wave_batch_kernel<true, kServeSteps, ST, ROUND>
-                : wave_batch_kernel<false, kServeSteps, ST, ROUND>,
-            cta_bytes<5, kServeSteps, ST>()};
+template <bool ROUND> WaveBatchFn pick_batch(bool mrt) {
+    return mrt ? wave_batch_kernel<true, kServeSteps, ROUND>
+               : wave_batch_kernel<false, kServeSteps, ROUND>;
 }
-WaveBatchPick pick_batch_f32(bool mrt);               // wave.cu
-WaveBatchPick pick_batch_bf16(bool mrt, bool round);  // wave_bf16.cu
+WaveBatchFn pick_batch_fp32(bool mrt);   // wave.cu: BF16 shots keep FP32 between a launch's steps
+WaveBatchFn pick_batch_round(bool mrt);  // wave_bf16.cu: they round at every step
 
 }  // namespace lbwave
