@@ -231,11 +231,11 @@ static long long tile_cost(const lb_ctx *c, int K) {
 // faster (2048^2: 10.8 against 11.0 us a step, 4096^2: 29 against 44).
 Fuse fuse_steps(const lb_ctx *c, int n) {
     const long long sites = (long long)c->ny * c->pitch;
-    if (c->Q == 5 && sites < 3500000) {
     // FP16: two, since its range scales are guessed no further ahead (a launch, the scale update and
     // a second launch that mostly ends at once; 3001 x 1777: 25.5 us a step against 35.9)
     if (c->cfg.storage == LB_F16)
         return Fuse{n >= 2 && wave_pays(c) ? 2 : 1, false};
+    if (c->Q == 5 && sites < 3500000) {
         if (n < 2) return Fuse{1, false};
         int best = 2;
         long long cost = -1;
@@ -271,17 +271,17 @@ lb_status tb_launch(lb_ctx *ctx, Fuse f) {
                       ? ctx->trace + row * ctx->nrec : nullptr;
     a.rho_out = tape_row(ctx, ctx->t);  // level j at rho_out + j plane
     a.rho_stride = (long long)ctx->ny * ctx->pitch;
+    if (ctx->lp_scale) f16_slots(ctx, a, K);
     lb_status st = ctx->cfg.storage == LB_BF16 && ctx->cfg.time_block > 1
                        ? tb5_launch_args(ctx, a, K)
-    if (ctx->lp_scale) f16_slots(ctx, a, K);
                        : fuse_launch_args(ctx, a, f);
-    if (st != LB_OK) return st;
-    ctx->cur ^= 1;
     if (st == LB_OK && ctx->lp_scale && (st = f16_update(ctx, a)) == LB_OK) {
         a.redo = f16_redo(ctx);  // once more, where the second step's scale was another
         ctx->n_launch++;
         st = fuse_launch_args(ctx, a, f);
     }
+    if (st != LB_OK) return st;
+    ctx->cur ^= 1;
     ctx->t += K;
     return LB_OK;
 }

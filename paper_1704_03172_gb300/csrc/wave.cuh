@@ -156,7 +156,6 @@ template <> struct Two<__nv_bfloat16> {
     __device__ static __forceinline__ float2 round(float2 v) { return unpack(pack(v)); }
 };
 
-// the values at x - 1 and x + 1 of a lane's columns
 template <> struct Two<__half> {
     __device__ static __forceinline__ uint32_t pack(float2 a) {
         const __half2 h = __floats2half2_rn(a.x, a.y);
@@ -218,6 +217,7 @@ template <int Q> struct Range<Q, __half> {
     }
 };
 
+// the values at x - 1 and x + 1 of a lane's columns
 __device__ __forceinline__ float2 from_left(float2 h) {
     return make_float2(__shfl_up_sync(0xffffffffu, h.y, 1), h.x);
 }
@@ -763,8 +763,8 @@ __device__ __forceinline__ void sweep(const StepArgs &a, const WaveArgs &w, int 
     const bool sp = T.src || has_rec;
     const int next_end = __any_sync(0xffffffffu, T.split) ? 0 : min(a.ny, rend);
     int slot = 0;
-#pragma unroll 1
     Range<Q, ST> range(a);
+#pragma unroll 1
     for (int r = rbeg; r < rend; r += 2) {
         const int e = fast_end(r);
 #pragma unroll 1
@@ -777,8 +777,8 @@ __device__ __forceinline__ void sweep(const StepArgs &a, const WaveArgs &w, int 
         if (r + 1 >= rend) break;
         iterate<Q, CK, K, REC, ST, ROUND, false, 1>(a, w, T, S, at, range, r + 1, rend, next_end, slot, sp);
     }
-}
     range.fold(a, T.lane, T.own);
+}
 
 // resident CTAs per SM the registers are cut for
 template <int Q, int K, typename ST> constexpr int min_ctas() { return Q == 9 ? (K > 2 ? (sizeof(ST) == 4 ? 2 : 3) : 3) : K > 4 ? 3 : 4; }
@@ -790,9 +790,9 @@ __global__ void __launch_bounds__(kCtaThreads, min_ctas<Q, K, ST>())
     // finished ones SM by SM, and leave it unevenly spread (4096^2: 38.7 us a step against 38.1,
     // 256^2: 3.1 against 2.5).
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    extern __shared__ __align__(16) unsigned char smem[];
     if constexpr (sizeof(ST) == 2 && K == 2)
         if (a.redo && *a.redo == 0u) return;  // (grid-uniform; FP16 only)
+    extern __shared__ __align__(16) unsigned char smem[];
     float *tab = reinterpret_cast<float *>(smem + kWarpsPerCta * warp_bytes<Q, K, ST>());
     const int wi = threadIdx.x >> 5;
     sweep<Q, CK, K, REC, ST, ROUND>(a, w, blockIdx.x * kWarpsPerCta + wi, smem + wi * warp_bytes<Q, K, ST>(), tab);
