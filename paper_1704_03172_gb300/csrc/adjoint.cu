@@ -648,7 +648,7 @@ extern "C" lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *g
     // last one goes to `last` (when given); rho(t) goes to tape[t - from] (when given).
     // Several steps per launch where the fused kernel has them (not from a raw state): its
     // results are the one-step kernels', so a BF16 replay reproduces the forward run.
-    const bool fuse = wave_supported(ctx);
+    const bool fuse = wave_supported(ctx) && ctx->cfg.storage != LB_F16;
     lb_status rst = LB_OK;
     auto replay = [&](const void *in, bool raw, long long from, int n, void *last, bool record) {
         int x = 0;
@@ -691,7 +691,12 @@ extern "C" lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *g
             d.resid = resid;
             d.nrec = ctx->nrec;
             d.segs = segs4;
-            if (wave && m + 1 >= kAdj5Levels) {  // levels sa + m .. sa + m - K + 1, wavefront
+            const int Kt = wave ? tile_adj_levels(ctx, m + 1) : 0;
+            if (Kt > 0) {  // levels sa + m .. sa + m - Kt + 1 on tiles
+                const cudaError_t e = tile_adj_launch(ctx, a, d, d.rho, a.t, Kt);
+                if (e != cudaSuccess && rst == LB_OK) rst = cuda_fail(ctx, e, "tiled adjoint");
+                m -= Kt;
+            } else if (wave && m + 1 >= kAdj5Levels) {  // levels sa + m .. sa + m - K + 1, wavefront
                 const cudaError_t e =
                     adj5_launch(ctx, a, d, d.rho, a.t, row_off, row_x, row_id);
                 if (e != cudaSuccess && rst == LB_OK) rst = cuda_fail(ctx, e, "wavefront adjoint");

@@ -150,3 +150,9 @@ void adj5_row_lists(const lb_ctx *ctx, std::vector<int> &off, std::vector<int> &
 cudaError_t adj5_launch(lb_ctx *ctx, const lbk::StepArgs &a, const lbadj::AdjArgs &d,
                         const float *rho_hi, long long t_hi, const int *row_off, const int *rec_x,
                         const int *rec_id);
+
+// The same on register tiles (tile_adj.cu): levels of the next launch of n wanted ones (0: the
+// grid is the wavefront's), and the launch of K levels
+int tile_adj_levels(const lb_ctx *ctx, int n);
+cudaError_t tile_adj_launch(lb_ctx *ctx, const lbk::StepArgs &a, const lbadj::AdjArgs &d,
+                            const float *rho_hi, long long t_hi, int K);

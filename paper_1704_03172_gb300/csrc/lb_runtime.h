@@ -127,6 +127,7 @@ void f16_slots(lb_ctx *ctx, lbk::StepArgs &a, int steps);
 lb_status f16_update(lb_ctx *ctx, const lbk::StepArgs &a);  // and the scales after it
 unsigned *f16_redo(const lb_ctx *ctx);
 int round_up(int v, int m);
+int sm_count();
 // scale pointers of the current buffer (nullptr for FP32 storage)
 const float *current_scale(const lb_ctx *ctx);
 lb_status fail(lb_ctx *ctx, lb_status st, const char *fmt, ...);

@@ -238,3 +238,36 @@ def test_tape_from_the_staged_step(sim_cls, oracle_mod, Q):
     assert rel(gs, os_) < TOL
     assert rel(gg, og) < TOL
     assert rel(gc, oc) < 4e-2
+
+
+# Up to 3.5 million sites the levels run on register tiles (csrc/tile_adj.cu): one tile, tiles that
+# end one column past the last, periodic grids smaller than a region, more tiles than SMs, several
+# receivers at a site and the source at one, and level counts that leave every remainder
+@pytest.mark.parametrize("coll,tau", [("bgk", 0.5), ("bgk", 0.8), ("mrt", 0.5)])
+@pytest.mark.parametrize("periodic", [False, True])
+@pytest.mark.parametrize("nx,ny,steps", [(33, 32, 9), (65, 57, 17), (121, 50, 12), (801, 700, 11)])
+def test_tiled_adjoint(sim_cls, oracle_mod, coll, tau, periodic, nx, ny, steps):
+    rng = np.random.default_rng(nx + steps)
+    c = W.random_medium(nx, ny, 3, 0.5, 1.0)
+    s = W.mrt_rates(5, W.DEFAULT_SEED + 2)
+    rec = np.stack([rng.integers(0, nx, 20), rng.integers(0, ny, 20)], 1).astype(np.int32)
+    src = (nx // 3, ny // 2, rng.normal(size=steps))
+    rec[0], rec[1], rec[2], rec[3] = src[:2], src[:2], (0, 0), (nx - 1, ny - 1)
+    p0 = rng.normal(size=(ny, nx)).astype(np.float32)
+    dj = rng.normal(size=(steps, len(rec))).astype(np.float32)
+    sponge = 0 if periodic else 5
+    sim = sim_cls(c.astype(np.float32), lattice=5, collision=coll, tau=tau, s=s, c_ref=1.0,
+                  boundary="periodic" if periodic else "zero", sponge_width=sponge)
+    sim.set_source(*src)
+    sim.set_receivers(rec, steps)
+    sim.init_pressure(p0)
+    sim.record_rho(steps)
+    sim.step(steps)
+    out = [x.cpu().numpy() for x in sim.adjoint(dj, steps, want_g0=True)]
+    sim.close()
+    P = oracle_mod.Problem(5, nx, ny, c.astype(np.float32), c_ref=1.0, tau=tau, mrt=coll == "mrt", s=s,
+                           periodic=periodic, sponge_width=sponge, sponge_sigma_max=0.1, source=src,
+                           receivers=rec)
+    ref = oracle_mod.adjoint(P, oracle_mod.init_pressure(P, p0.astype(np.float64)), steps, dj.astype(np.float64))
+    for a, b in zip(out, ref):
+        assert np.linalg.norm(a - b) <= TOL * np.linalg.norm(b)
