@@ -107,8 +107,8 @@ typedef struct {
                                  at a time.  D2Q5: 2, 4, 6, 8 or 16 with FP32 or BF16 storage
                                  (BF16: whole blocks, FP32 between their steps); D2Q9: 2 or 4
                                  with FP32 storage.  <= 1: lb_step fuses steps by itself where
-                                 that is faster and changes nothing: with LB_STEP_AUTO, on 2-D
-                                 FP32 / BF16 grids without patch, slab or in-place streaming, the
+                                 that is faster and changes nothing: with LB_STEP_AUTO, on grids
+                                 without patch, slab or in-place streaming (FP16: D2Q5 only), the
                                  results equal one launch per step bit for bit */
     /* Optional device allocator (e.g. PyTorch's caching allocator).  NULL: cudaMalloc. */
     void *(*dev_alloc)(size_t bytes, void *user);
@@ -443,7 +443,8 @@ lb_status lb_mode_projection(lb_ctx *ctx, const int *modes, int n_modes, double 
  * dt = dx c_s(eta=1) / c_ref (seconds; 0 when dx or c_ref is 0), info[4] = number
  * of distinct speeds when the step reads a 1-byte medium index (host c_map with at
  * most 256 distinct values), 0 when it reads eta^2 per site, info[5] = 1 when a step
- * runs the TMA-staged persistent kernel, else 0.  Fills min(n_info, 6) entries. */
+ * runs the TMA-staged persistent kernel, else 0, info[6] = kernels that lb_step has launched
+ * on this context (uniform two-buffer grids).  Fills min(n_info, 7) entries. */
 lb_status lb_info(const lb_ctx *ctx, double *info, int n_info);
 
 const char *lb_last_error(const lb_ctx *ctx);

@@ -147,7 +147,7 @@ __global__ void adjoint_receivers(const StepArgs a, const AdjArgs d) {
 
 // ---- time-blocked reverse sweep: K adjoint levels per launch
 //
-// The transpose of the overlapped tiling of tblock.cu.  A CTA owns an OUT x OUT tile
+// The transpose of an overlapped tiling of several steps.  A CTA owns an OUT x OUT tile
 // (OUT = 48 - 2K) and loads lambda^{t_hi+1} on the 48 x 48 region made of the tile and a
 // K-site halo; level j (time t = t_hi - j) turns lambda^{t+1} into lambda^t in shared
 // memory for every site whose distance to the region edge exceeds j (its pull from

@@ -34,7 +34,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kSitesPerWarp = 128;       // 32 lanes x 4 sites
 static_assert(kThreads == 256, "one medium-table entry per thread");
 
-// Time-blocked kernels (tblock.cu forward, adjoint.cu reverse): one CTA of kTbThreads
+// Time-blocked kernels (adjoint.cu reverse): one CTA of kTbThreads
 // threads per kTbW x kTbW region (an output tile plus a K-site halo), each thread
 // holding the same kTbPer sites of the region for every level.
 constexpr int kTbW = 48;

@@ -180,7 +180,11 @@ bool wave_supported(const lb_ctx *ctx);
 Fuse fuse_steps(const lb_ctx *ctx, int n);
 lb_status wave_set_receivers(lb_ctx *ctx, const int *xy, int nrec);
 lb_status fuse_launch_args(lb_ctx *ctx, const lbk::StepArgs &a, Fuse f);
-// its served batches of D2Q5 shots, kServeSteps steps per launch: staging bytes of one launch's
+// two fused D3Q7 steps (sweep3.cu), FP32 or BF16, bit for bit the one-step results
+bool sweep3_supported(const lb_ctx *ctx);
+bool sweep3_pays(const lb_ctx *ctx);
+lb_status sweep3_launch(lb_ctx *ctx, const lbk::StepArgs &a);
+// the wavefront's served batches of D2Q5 shots, kServeSteps steps per launch: staging bytes of one launch's
 // descriptors, whether a shot can take the steps now, the rows per warp that suit n shots
 // together, a shot's CTAs at H rows per warp, the fill (advancing the shots) and the launch from
 // the device copy of the staging block.  BF16 shots round at every step, as the one-step

@@ -1066,7 +1066,8 @@ static Fuse next_launch(const lb_ctx *ctx, int left) {
     if (T > 1 && ctx->cfg.storage == LB_BF16)  // FP32 between the levels: no rho record
         return room >= T && !taping ? Fuse{T, false} : one;
     if (T > 1) return fuse_steps(ctx, (int)std::min<long long>(room, T));
-    if (ctx->cfg.step_kernel != LB_STEP_AUTO || !wave_supported(ctx)) return one;
+    if (ctx->cfg.step_kernel != LB_STEP_AUTO || !(wave_supported(ctx) || sweep3_supported(ctx)))
+        return one;
     return fuse_steps(ctx, (int)std::min<long long>(room, 1 << 20));
 }
 
@@ -1087,6 +1088,7 @@ static lb_status step_n(lb_ctx *ctx, int n) {
         const Fuse f = next_launch(ctx, n - k);
         lb_status st = f.steps > 1 ? tb_launch(ctx, f) : launch_step(ctx, fn, a);
         if (st != LB_OK) return st;
+        ctx->n_launch++;
         k += f.steps;
     }
     return check_launch(ctx, "step_kernel");
@@ -1135,7 +1137,7 @@ lb_status lb_sync(lb_ctx *ctx) {
 
 lb_status lb_info(const lb_ctx *ctx, double *info, int n_info) {
     if (!ctx || !info) return LB_EINVAL;
-    double v[6];
+    double v[7];
     v[0] = ctx->Q;
     v[1] = ctx->pitch;
     v[2] = ctx->ebytes;
@@ -1144,7 +1146,8 @@ lb_status lb_info(const lb_ctx *ctx, double *info, int n_info) {
     v[3] = (ctx->cfg.dx > 0 && ctx->cfg.c_ref > 0) ? ctx->cfg.dx * cs_ref / ctx->cfg.c_ref : 0.0;
     v[4] = ctx->n_mid;
     v[5] = ctx->staged ? 1.0 : 0.0;
-    for (int k = 0; k < n_info && k < 6; k++) info[k] = v[k];
+    v[6] = (double)ctx->n_launch;
+    for (int k = 0; k < n_info && k < 7; k++) info[k] = v[k];
     return LB_OK;
 }
 

@@ -206,6 +206,7 @@ static lb_status tile_launch(lb_ctx *ctx, const StepArgs &a, const WaveArgs &rec
 // f.steps fused steps with the caller's arguments (a.in must not be raw); receivers when
 // a.trace_row is set and the row lists exist; rho of every level when a.rho_out is set.
 lb_status fuse_launch_args(lb_ctx *ctx, const StepArgs &a, Fuse f) {
+    if (ctx->Q == 7) return sweep3_launch(ctx, a);
     WaveArgs w = {};
     w.row_off = a.trace_row ? ctx->row_off : nullptr;
     w.rec_x = ctx->row_x;
@@ -231,6 +232,7 @@ static long long tile_cost(const lb_ctx *c, int K) {
 // faster (2048^2: 10.8 against 11.0 us a step, 4096^2: 29 against 44).
 Fuse fuse_steps(const lb_ctx *c, int n) {
     const long long sites = (long long)c->ny * c->pitch;
+    if (c->Q == 7) return Fuse{n >= 2 && sweep3_pays(c) ? 2 : 1, false};
     // FP16: two, since its range scales are guessed no further ahead (a launch, the scale update and
     // a second launch that mostly ends at once; 3001 x 1777: 25.5 us a step against 35.9)
     if (c->cfg.storage == LB_F16)
@@ -267,7 +269,7 @@ lb_status tb_launch(lb_ctx *ctx, Fuse f) {
     a.t = ctx->t;
     a.raw = 0;
     const long long row = ctx->t - ctx->t_rec0;
-    a.trace_row = (ctx->trace && ctx->row_off && row >= 0 && row + K <= ctx->trace_cap)
+    a.trace_row = (ctx->trace && (ctx->row_off || ctx->Q == 7) && row >= 0 && row + K <= ctx->trace_cap)
                       ? ctx->trace + row * ctx->nrec : nullptr;
     a.rho_out = tape_row(ctx, ctx->t);  // level j at rho_out + j plane
     a.rho_stride = (long long)ctx->ny * ctx->pitch;

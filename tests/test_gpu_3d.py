@@ -122,3 +122,41 @@ def test_d3q7_staged_step_matches_direct_bitwise(sim_cls, storage, periodic, nx,
         sim.close()
     np.testing.assert_array_equal(out[0][0], out[1][0])
     np.testing.assert_array_equal(out[0][1], out[1][1])
+
+
+# Two steps per launch (csrc/sweep3.cuh), on grids just large enough for them, against one, bit for
+# bit: one tile and several, sides one past a tile's and a warp's, chunks of one plane, widths that
+# end in half a lane, odd periodic seams, periodic grids smaller than a region, receivers on faces
+# and more than one block of them, a source at a tile's edge and at the wrap, an odd number of steps
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("periodic", [False, True])
+@pytest.mark.parametrize("nx,ny,nz", [(3, 310, 310), (57, 31, 1600), (60, 30, 1570), (61, 61, 780),
+                                      (64, 24000, 2), (129, 94, 210), (257, 33, 320), (1100, 15, 180)])
+def test_fused_steps_match_direct_bitwise(sim_cls, storage, periodic, nx, ny, nz):
+    import torch
+    rng = np.random.default_rng(nx + ny)
+    steps = 8
+    gen = torch.Generator(device="cuda").manual_seed(nx)
+    g0 = torch.randn((7, nz, ny, nx), generator=gen, device="cuda")
+    rec = np.stack([rng.integers(0, nx, 700), rng.integers(0, ny, 700), rng.integers(0, nz, 700)],
+                   1).astype(np.int32)
+    rec[0], rec[1], rec[2] = 0, (nx - 1, ny - 1, nz - 1), (nx // 2, 0, nz - 1)
+    wav = rng.normal(size=steps - 2)
+    for layered, tau, sponge, src in ((True, 0.5, 0, (0, 0, 0)), (False, 0.8, 2, (nx - 1, ny // 2, nz - 1)),
+                                      (False, 0.5, 0 if periodic else 5, (nx // 2, min(ny - 1, 30), nz // 2))):
+        c = (_layered3(nx, ny, nz) if layered
+             else 0.45 + 0.55 * torch.rand((nz, ny, nx), generator=gen, device="cuda"))
+        out = []
+        for how in ("direct", "auto"):
+            sim = sim_cls(c, lattice=7, tau=tau, storage=storage, c_ref=1.0, step_kernel=how,
+                          boundary="periodic" if periodic else "zero", sponge_width=sponge)
+            sim.set_source(*src, wav)
+            sim.set_receivers(rec, steps)
+            sim.set_state(g0)
+            before = sim.info()[6]
+            sim.step(steps)
+            assert sim.info()[6] - before == (steps if how == "direct" else 1 + 3 + 1)
+            out.append((sim.state().clone(), sim.traces(steps).clone()))
+            sim.close()
+        assert torch.equal(out[0][0], out[1][0])
+        assert torch.equal(out[0][1], out[1][1])
