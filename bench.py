@@ -940,6 +940,7 @@ def run_ours(args):
     wl["step_kernel"] = args.step_kernel
     sim = _make_sim(LBSim, wl, args.steps + args.warmup)
     sim.step(args.warmup)
+    launches = sim.info()[6]
     torch.cuda.synchronize()
     if ws > 1:
         dist.barrier()
@@ -961,6 +962,7 @@ def run_ours(args):
     tr = sim.traces(args.steps + args.warmup)
     finite = bool(torch.isfinite(tr).all().item())
     indexed = _indexed(sim)
+    launches = int(sim.info()[6] - launches)
     sim.close()
     value = rate / 1e9
     if rank != 0:
@@ -968,21 +970,16 @@ def run_ours(args):
             dist.destroy_process_group()
         return 0
     peak, peak_kind = _peaks()
-    K = max(1, args.time_block)
-    # the one-step and the D2Q5 wavefront kernels read the 1-byte medium index; the D2Q9
-    # tile-blocked kernel reads eta^2 per site
-    medium_idx = indexed and (K == 1 or args.lattice == 5)
-    bps = bytes_per_site(args.lattice, args.storage, medium_idx)
-    launches = (args.steps + K - 1) // K
-    per_launch_s = sec / launches
-    achieved = bps * sites * K / per_launch_s / 1e9   # algorithmic one-step bytes per update
-    staged = K == 1 and (args.step_kernel == "staged" or
-                         (args.step_kernel == "auto" and args.storage != "f32"))
+    # lb_step takes several steps per launch where its fused kernels are faster
+    fused = args.steps / max(launches, 1)
+    bps = bytes_per_site(args.lattice, args.storage, indexed)
+    achieved = bps * sites * args.steps / sec / 1e9   # algorithmic one-step bytes per update
+    staged = (args.step_kernel == "staged" or
+              (args.step_kernel == "auto" and args.storage != "f32"))
     st_name = dict(f32='float', bf16='__nv_bfloat16', f16='__half')[args.storage]
     mrt = "true" if args.collision == "mrt" else "false"
-    tb5 = K > 1 and args.lattice == 5
-    kname = (f"lbtb5::tb5_kernel<{mrt},{K},false,{st_name}>" if tb5 else
-             f"tb_kernel<{args.lattice},{mrt},false,{K}>" if K > 1 else
+    kname = ("lbtb5::tb5_kernel" if args.time_block > 1 and args.storage == "bf16" else
+             "lbwave::wave_kernel" if fused > 1 else
              f"stream_step_kernel<{args.lattice},{mrt},false,{st_name}>" if staged else
              f"lbk::step_kernel<{args.lattice},{mrt},false,{st_name}>")
     traffic, traffic_src = ncu_traffic(kname, indexed)
@@ -996,18 +993,18 @@ def run_ours(args):
                                                          else "MRT (seeded rates)") +
                                f", {args.storage.upper()} populations, "
                                "40-cell sponge, Ricker source, 512 receivers; one bench step = "
-                               "one LB time step" + (f" ({K} steps fused per launch)" if K > 1 else ""),
+                               "one LB time step" + (f" ({fused:.1f} steps fused per launch)" if fused > 1 else ""),
                    "parallelism": f"replicas x{ws} (independent shots)",
                    "l2": "inputs larger than L2 (each population buffer >= 168 MB; 129 MB L2)",
-                   "medium": "1-byte medium index + eta^2 table" if medium_idx
+                   "medium": "1-byte medium index + eta^2 table" if indexed
                              else "eta^2 per site (FP32)"},
         "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak,
                      "peak_kind": peak_kind, "unit": "GB/s", "frac": round(achieved / peak, 4),
                      "traffic": traffic, "traffic_source": traffic_src, "kernel": kname,
-                     "algorithmic_bytes_per_launch": bps * sites * K,
+                     "algorithmic_bytes_per_launch": round(bps * sites * fused),
                      "note": "achieved counts the one-step algorithmic bytes of every fused "
                              "step (one-step equivalent bandwidth)"
-                     if K > 1 else "one launch per step"},
+                     if fused > 1 else "one launch per step"},
         "gpu_launches": launches,
         "clocks": clk.summary(),
         "wall_s": round(wall, 4),
