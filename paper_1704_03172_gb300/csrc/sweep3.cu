@@ -19,8 +19,10 @@ bool sweep3_supported(const lb_ctx *c) {
 // Where both states stay in L2 the one-step kernels are as fast or faster (us a step, one / two per
 // launch: FP32 96^3 10.2 / 11.5, 128^3 20.2 / 21.5, 192^3 74.8 / 55.4, 320^3 309 / 212; BF16, whose
 // one-step kernel converts twice as often: 64^3 8.5 / 8.7, 96^3 15.0 / 11.9, 128^3 24.6 / 21.0; staged
-// (1100 x 40 x 40) 13.3 / 15.7, 320^3 290 / 162).
+// (1100 x 40 x 40) 13.3 / 15.7, 320^3 290 / 162).  Odd periodic grids, whose rows are not whole
+// lanes at the seam, keep single steps too.
 bool sweep3_pays(const lb_ctx *c) {
+    if (c->cfg.boundary == LB_PERIODIC && c->nx % 2 != 0) return false;
     return (long long)c->ny * c->pitch >= (c->cfg.storage == LB_BF16 && !c->staged ? 800000 : 3000000);
 }
 

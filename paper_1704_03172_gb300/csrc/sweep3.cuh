@@ -87,44 +87,23 @@ __device__ __forceinline__ void issue(const StepArgs &a, const Lane &T, SharedZ<
                         wanted && yc >= 0 && zm >= 0, wanted && yc >= 0 && zp >= 0};
     const int ys[7] = {yc, yc, ym, yc, yp, yc, yc}, zs[7] = {zc, zc, zc, zc, zc, zm, zp};
     const ST *in = static_cast<const ST *>(a.in);
-    if (!T.split) {
-        const int x = T.live ? T.gxw : 0;
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sh.pop[row][0][2 * T.lane]);
+    const int x = T.live ? T.gxw : 0;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sh.pop[row][0][2 * T.lane]);
 #pragma unroll
-        for (int i = 0; i < 7; i++) {
-            const long long o = ok[i] ? (long long)(zs[i] * a.ny3 + ys[i]) * a.pitch : 0;
-            cp_async<2 * (int)sizeof(ST)>(dst + i * kRegX * (int)sizeof(ST), in + i * a.plane + o + x,
-                                          ok[i] && T.live);
-        }
-        const long long o = c ? (long long)(zc * a.ny3 + yc) * a.pitch : 0;
-        const uint32_t med = (uint32_t)__cvta_generic_to_shared(&sh.med[row][T.lane]);
-        if (a.mid)
-            cp_async<4>(med, a.mid + o + (x & ~3), c && T.live);
-        else
-            cp_async<8>(med, a.eta2 + o + x, c && T.live);
-        return;
+    for (int i = 0; i < 7; i++) {
+        const long long o = ok[i] ? (long long)(zs[i] * a.ny3 + ys[i]) * a.pitch : 0;
+        cp_async<2 * (int)sizeof(ST)>(dst + i * kRegX * (int)sizeof(ST), in + i * a.plane + o + x,
+                                      ok[i] && T.live);
     }
-    // the lanes at a periodic seam, column by column (every row and plane exists)
-    unsigned w = 0;
-#pragma unroll 1
-    for (int j = 0; j < 2; j++) {
-        const int x = wrap1(T.gx + j, a.nx);
-#pragma unroll 1
-        for (int i = 0; i < 7; i++) {
-            const int r = (i == 5 ? zm : i == 6 ? zp : zc) * a.ny3 + (i == 2 ? ym : i == 4 ? yp : yc);
-            sh.pop[row][i][2 * T.lane + j] = in[i * a.plane + (long long)r * a.pitch + x];
-        }
-        const long long p = (long long)(zc * a.ny3 + yc) * a.pitch + x;
-        if (a.mid)
-            w |= (unsigned)a.mid[p] << (8 * j);
-        else
-            reinterpret_cast<float *>(&sh.med[row][T.lane])[j] = a.eta2[p];
-    }
-    // (placed as the aligned word of an unsplit lane would hold the two bytes)
-    if (a.mid) reinterpret_cast<unsigned *>(&sh.med[row][T.lane])[0] = w << (8 * (T.gxw & 2));
+    const long long o = c ? (long long)(zc * a.ny3 + yc) * a.pitch : 0;
+    const uint32_t med = (uint32_t)__cvta_generic_to_shared(&sh.med[row][T.lane]);
+    if (a.mid)
+        cp_async<4>(med, a.mid + o + (x & ~3), c && T.live);
+    else
+        cp_async<8>(med, a.eta2 + o + x, c && T.live);
 }
 
-// The same for lanes that have their two columns next to each other, where no row or plane wraps.
+// The same where no row, plane or column wraps.
 // at0: row y's first value in plane z (the same for all lanes); lane: the lane's columns from there.
 // CHECK: rows and planes may lie outside a zero-ghost grid; otherwise they all lie inside.
 template <typename ST, bool CHECK>
@@ -373,11 +352,9 @@ __global__ void __launch_bounds__(kThreadsZ, 2) sweep3_kernel(const StepArgs a, 
     const int y0 = ylo - kHaloY + v * kRowsZ;
     T.gx = xlo - kHaloX + 2 * T.lane;
     T.gxw = T.gx;
-    T.split = false;
     T.live = T.gx <= xhi + 1;  // level 1 of column xhi pulls from xhi + 1
     if (T.per) {
-        T.gxw = wrap1(T.gx, a.nx);
-        T.split = T.live && ((T.gxw & 1) != 0 || T.gxw + 1 >= a.nx);
+        T.gxw = wrap1(T.gx, a.nx);  // (nx is even: a lane's columns stay together)
     } else {
         T.live = T.live && T.gx >= 0 && T.gx < a.nx;
     }
@@ -426,7 +403,7 @@ __global__ void __launch_bounds__(kThreadsZ, 2) sweep3_kernel(const StepArgs a, 
     const int from = T.live ? lane : y0 * a.pitch;  // where it copies from (nothing if not live)
     // rows inside with those next to them (the rows beyond the tile's are copied too)
     const bool rows_in = y0 >= 1 && y0 + kRowsZ < a.ny3;
-    const bool whole = !T.per || (rows_in && !__any_sync(0xffffffffu, T.split || T.gx != T.gxw));
+    const bool whole = !T.per || (rows_in && !__any_sync(0xffffffffu, T.gx != T.gxw));
     const bool out = !T.per && (xlo == 0 || xhi >= a.nx || ylo == 0 || yhi >= a.ny3);
     const bool pad = xhi == a.nx && (a.nx & 1) != 0;
 #pragma unroll 1

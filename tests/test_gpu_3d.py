@@ -126,11 +126,11 @@ def test_d3q7_staged_step_matches_direct_bitwise(sim_cls, storage, periodic, nx,
 
 # Two steps per launch (csrc/sweep3.cuh), on grids just large enough for them, against one, bit for
 # bit: one tile and several, sides one past a tile's and a warp's, chunks of one plane, widths that
-# end in half a lane, odd periodic seams, periodic grids smaller than a region, receivers on faces
+# end in half a lane, periodic grids smaller than a region, receivers on faces
 # and more than one block of them, a source at a tile's edge and at the wrap, an odd number of steps
 @pytest.mark.parametrize("storage", ["f32", "bf16"])
 @pytest.mark.parametrize("periodic", [False, True])
-@pytest.mark.parametrize("nx,ny,nz", [(3, 310, 310), (57, 31, 1600), (60, 30, 1570), (61, 61, 780),
+@pytest.mark.parametrize("nx,ny,nz", [(3, 310, 310), (58, 31, 1600), (57, 31, 1600), (60, 30, 1570), (61, 61, 780),
                                       (64, 24000, 2), (129, 94, 210), (257, 33, 320), (1100, 15, 180)])
 def test_fused_steps_match_direct_bitwise(sim_cls, storage, periodic, nx, ny, nz):
     import torch
@@ -155,7 +155,8 @@ def test_fused_steps_match_direct_bitwise(sim_cls, storage, periodic, nx, ny, nz
             sim.set_state(g0)
             before = sim.info()[6]
             sim.step(steps)
-            assert sim.info()[6] - before == (steps if how == "direct" else 1 + 3 + 1)
+            one = how == "direct" or (periodic and nx % 2)  # odd periodic rows keep single steps
+            assert sim.info()[6] - before == (steps if one else 1 + 3 + 1)
             out.append((sim.state().clone(), sim.traces(steps).clone()))
             sim.close()
         assert torch.equal(out[0][0], out[1][0])

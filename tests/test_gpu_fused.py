@@ -96,7 +96,7 @@ def test_tiles(sim_cls, coll, tau, storage, boundary):
 @pytest.mark.parametrize("boundary", ["zero", "periodic"])
 def test_f16_two_steps(sim_cls, coll, tau, boundary):
     import torch
-    for nx, ny, sponge in ((57, 2600, 6), (601, 300, 0), (1531, 117, 9)):
+    for nx, ny, sponge in ((1031, 489, 6), (1100, 460, 0), (2051, 250, 9)):
         rng = np.random.default_rng(nx)
         c = W.random_medium(nx, ny, 5, 0.5, 1.0).astype(np.float32)
         steps = 28
