@@ -67,6 +67,11 @@ __device__ __forceinline__ void collide7p(float2 (&g)[7], float2 e2, float om) {
     g[6] = relax(fma(-0.5f, jz, b), g[6]);
 }
 
+// First value of row y of plane z.  64 bits throughout: a plane alone may hold more than 2^31 sites.
+__host__ __device__ constexpr long long row_start(int y, int z, int ny3, int pitch) {
+    return ((long long)z * ny3 + y) * pitch;
+}
+
 // index of a row or plane in the grid: wrapped, or -1 outside a zero-ghost grid
 __device__ __forceinline__ int at_or_none(int v, int n, bool per) {
     return per ? wrap1(v, n) : (unsigned)v < (unsigned)n ? v : -1;
@@ -91,11 +96,11 @@ __device__ __forceinline__ void issue(const StepArgs &a, const Lane &T, SharedZ<
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sh.pop[row][0][2 * T.lane]);
 #pragma unroll
     for (int i = 0; i < 7; i++) {
-        const long long o = ok[i] ? (long long)(zs[i] * a.ny3 + ys[i]) * a.pitch : 0;
+        const long long o = ok[i] ? row_start(ys[i], zs[i], a.ny3, a.pitch) : 0;
         cp_async<2 * (int)sizeof(ST)>(dst + i * kRegX * (int)sizeof(ST), in + i * a.plane + o + x,
                                       ok[i] && T.live);
     }
-    const long long o = c ? (long long)(zc * a.ny3 + yc) * a.pitch : 0;
+    const long long o = c ? row_start(yc, zc, a.ny3, a.pitch) : 0;
     const uint32_t med = (uint32_t)__cvta_generic_to_shared(&sh.med[row][T.lane]);
     if (a.mid)
         cp_async<4>(med, a.mid + o + (x & ~3), c && T.live);
@@ -104,12 +109,12 @@ __device__ __forceinline__ void issue(const StepArgs &a, const Lane &T, SharedZ<
 }
 
 // The same where no row, plane or column wraps.
-// at0: row y's first value in plane z (the same for all lanes); lane: the lane's columns from there.
+// at0: row y's first value in plane z (the same for all lanes); lane: the lane's columns in the row.
 // CHECK: rows and planes may lie outside a zero-ghost grid; otherwise they all lie inside.
 template <typename ST, bool CHECK>
 __device__ __forceinline__ void issue_inside(const StepArgs &a, const Lane &T, SharedZ<ST> &sh, int row,
                                              int y, int z, long long at0, int lane) {
-    const long long dz = (long long)a.ny3 * a.pitch;
+    const long long dz = row_start(0, 1, a.ny3, a.pitch);
     const long long by[7] = {0, 0, -(long long)a.pitch, 0, a.pitch, -dz, dz};
     bool c = T.live, ok[7] = {c, c, c, c, c, c, c};
     if (CHECK) {
@@ -398,9 +403,8 @@ __global__ void __launch_bounds__(kThreadsZ, 2) sweep3_kernel(const StepArgs a, 
         for (int i = 0; i < 5; i++) H[j][i] = f2(0.f);
     }
     const int sz = a.src_y / a.ny3;
-    const long long dz = (long long)a.ny3 * a.pitch;
-    const int lane = y0 * a.pitch + T.gx;  // the lane's columns of the warp's first row, in a plane
-    const int from = T.live ? lane : y0 * a.pitch;  // where it copies from (nothing if not live)
+    const int lane = T.gx;               // the lane's columns in a row
+    const int from = T.live ? lane : 0;  // where it copies from (nothing if not live)
     // rows inside with those next to them (the rows beyond the tile's are copied too)
     const bool rows_in = y0 >= 1 && y0 + kRowsZ < a.ny3;
     const bool whole = !T.per || (rows_in && !__any_sync(0xffffffffu, T.gx != T.gxw));
@@ -420,13 +424,16 @@ __global__ void __launch_bounds__(kThreadsZ, 2) sweep3_kernel(const StepArgs a, 
                 s0 = at_or_none(z - 1, a.nz, T.per) == sz ? src_rows : 0u;
             }
             const bool ghost = out || (!T.per && (z - 1 < 0 || z >= a.nz));
+            // the warp's first row in planes z + 1 and z - 1
+            const long long up0 = row_start(y0, z + 1, a.ny3, a.pitch),
+                            down0 = row_start(y0, z - 1, a.ny3, a.pitch);
             if (rows == 0) {  // warp-uniform
             } else if (edge || (s1 | s0))
-                plane<ST, kEdges>(a, T, sh, H, H5, v, y0, z, next && z < zhi, (z + 1) * dz, from, z - 1 >= zlo,
-                                  (z - 1) * dz, lane, own_rows, ghost, s1, s0);
+                plane<ST, kEdges>(a, T, sh, H, H5, v, y0, z, next && z < zhi, up0, from, z - 1 >= zlo,
+                                  down0, lane, own_rows, ghost, s1, s0);
             else
-                plane<ST, kInside>(a, T, sh, H, H5, v, y0, z, next && z < zhi, (z + 1) * dz, from, z - 1 >= zlo,
-                                   (z - 1) * dz, lane, own_rows, false, 0u, 0u);
+                plane<ST, kInside>(a, T, sh, H, H5, v, y0, z, next && z < zhi, up0, from, z - 1 >= zlo,
+                                   down0, lane, own_rows, false, 0u, 0u);
         }
         if (rows && z < zhi && !(next && z >= zlo - 1)) {
 #pragma unroll 1
