@@ -6,6 +6,8 @@
 // shuffle, rows beyond the warp's four through shared memory, one barrier a level.  rho of the
 // next level comes by cp.async while this one is computed.  The medium gradient's terms are
 // summed in FP32 over four levels at a time, as the wavefront sums them, and in FP64 from there.
+// The levels that are left over where four do not divide a sweep are multiplied and summed in
+// FP64 (WIDE), as the one-level kernel (adjoint.cu) does: a sum of few terms may cancel.
 //
 // What bounds it and why this shape: issue, and the barrier.  A wavefront launch takes its rows one
 // after another and needs 2 K of them to start with, which small grids cannot hide.  1201 x 911
@@ -14,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "adjoint_site.cuh"
 #include "lb_kernels.cuh"
@@ -40,7 +43,10 @@ struct SharedAdj {
     float2 e2[kSide][32];               // eta^2; from here on read by the lane that wrote it
     float2 factor[kSide][32];           // sponge factors (0 outside a zero-ghost grid)
     float2 rho[kSide][32];              // rho of the next level (own sites; else 0)
-    float2 sum[2][kSide][32];           // gradient terms of levels 0 .. 3 and 4 .. 7
+    union {
+        float2 sum[2][kSide][32];       // gradient terms of levels 0 .. 3 and 4 .. 7
+        double2 wide[kSide][32];        // WIDE: of all levels
+    };
     int2 rec[kSide][32];                // by column: receiver id, -1 none, -2 several
 };
 
@@ -93,34 +99,38 @@ __device__ __forceinline__ int receiver_at(const WaveArgs &w, int y, int x) {
     return e + 1 < hi && w.rec_x[e + 1] == x ? -2 : w.rec_id[e];
 }
 // the sum of dJ/dp over a site's receivers at row `row` of dJ/dp
-__device__ __forceinline__ float residual(const AdjArgs &d, const WaveArgs &w, int id, int y, int x,
-                                          long long row) {
-    if (id == -1) return 0.f;
+template <typename R>
+__device__ __forceinline__ R residual(const AdjArgs &d, const WaveArgs &w, int id, int y, int x,
+                                      long long row) {
+    if (id == -1) return 0;
     const float *p = d.resid + row * d.nrec;
     if (id >= 0) return p[id];
-    float R = 0.f;
+    R sum = 0;
     const int hi = w.row_off[y + 1];
-    for (int e = first_of(w, y, x); e < hi && w.rec_x[e] == x; e++) R += p[w.rec_id[e]];
-    return R;
+    for (int e = first_of(w, y, x); e < hi && w.rec_x[e] == x; e++) sum += p[w.rec_id[e]];
+    return sum;
 }
 
-template <bool MRT, int WHAT>
+template <bool MRT, int WHAT, bool WIDE>
 __device__ __forceinline__ void level(const StepArgs &a, const AdjArgs &d, const TileAdjArgs &w,
                                       const Lane &T, SharedAdj &sh, float2 (&h)[kRows][5], float2 up,
                                       float2 above, int y0, int l, unsigned own_rows,
                                       unsigned src_rows, unsigned rec_rows) {
     const int v = threadIdx.x >> 5;
     const long long t = w.t_hi - l;
-    float2 R[kRows];
+    using V = std::conditional_t<WIDE, double, float>;  // of a gradient term
+    struct {
+        V x, y;
+    } R[kRows];
     if (WHAT == kSpecial) {  // on their way while the rows before are computed
 #pragma unroll
         for (int j = 0; j < kRows; j++) {
-            R[j] = f2(0.f);
+            R[j].x = R[j].y = 0;
             if (rec_rows >> j & 1u) {  // warp-uniform
                 const int2 id = sh.rec[v * kRows + j][T.lane];
                 const int y = T.per ? wrap1(y0 + j, a.ny) : y0 + j;
-                R[j].x = residual(d, w.rec, id.x, y, col_of(T, a, 0), t - d.t0);
-                R[j].y = residual(d, w.rec, id.y, y, col_of(T, a, 1), t - d.t0);
+                R[j].x = residual<V>(d, w.rec, id.x, y, col_of(T, a, 0), t - d.t0);
+                R[j].y = residual<V>(d, w.rec, id.y, y, col_of(T, a, 1), t - d.t0);
             }
         }
     }
@@ -137,7 +147,12 @@ __device__ __forceinline__ void level(const StepArgs &a, const AdjArgs &d, const
         m[2] = j + 1 < kRows ? h[j + 1 < kRows ? j + 1 : 0][4] : above;
         up = h[j][2];
         const float2 e2 = sh.e2[row][T.lane], rho = sh.rho[row][T.lane];
-        float2 part = sh.sum[l >> 2][row][T.lane];
+        float2 part = f2(0.f);
+        double2 wide = make_double2(0., 0.);
+        if (WIDE)
+            wide = sh.wide[row][T.lane];
+        else
+            part = sh.sum[l >> 2][row][T.lane];
         if (WHAT != kPlain) {
             const float2 f = sh.factor[row][T.lane];
 #pragma unroll
@@ -152,18 +167,37 @@ __device__ __forceinline__ void level(const StepArgs &a, const AdjArgs &d, const
                 float src_w, src_dw;
                 adj_src<5>(mm, c ? e2.y : e2.x, a, src_w, src_dw);
                 if (T.own && T.gx + c < a.nx && (own_rows >> j & 1u)) d.grad_src[t - d.t0] = (double)src_w;
-                if (t < a.src_nt) (c ? part.y : part.x) += a.src_tab[t] * src_dw;
+                if (t < a.src_nt) {
+                    if (WIDE)
+                        (c ? wide.y : wide.x) += (double)a.src_tab[t] * (double)src_dw;
+                    else
+                        (c ? part.y : part.x) += a.src_tab[t] * src_dw;
+                }
             }
         }
         const float2 gsum = site<MRT>(m, e2, a);
-        part = fma2(rho, gsum, part);
+        if (WIDE) {
+            wide.x += (double)rho.x * (double)gsum.x;
+            wide.y += (double)rho.y * (double)gsum.y;
+        } else {
+            part = fma2(rho, gsum, part);
+        }
         if (WHAT == kSpecial && (rec_rows >> j & 1u)) {
-            const float2 Rc = make_float2(R[j].x * cs2_of<5>(e2.x, a), R[j].y * cs2_of<5>(e2.y, a));
+            const float2 R2 = make_float2((float)R[j].x, (float)R[j].y);
+            const float2 Rc = make_float2(R2.x * cs2_of<5>(e2.x, a), R2.y * cs2_of<5>(e2.y, a));
 #pragma unroll
             for (int i = 0; i < 5; i++) m[i] = add(m[i], Rc);
-            part = fma2(mul(R[j], f2(dcs2<5>(a))), rho, part);
+            if (WIDE) {
+                wide.x += (double)R[j].x * (double)dcs2<5>(a) * (double)rho.x;
+                wide.y += (double)R[j].y * (double)dcs2<5>(a) * (double)rho.y;
+            } else {
+                part = fma2(mul(R2, f2(dcs2<5>(a))), rho, part);
+            }
         }
-        sh.sum[l >> 2][row][T.lane] = part;
+        if (WIDE)
+            sh.wide[row][T.lane] = wide;
+        else
+            sh.sum[l >> 2][row][T.lane] = part;
         h[j][0] = m[0];
         h[j][1] = m[3];
         h[j][2] = m[4];
@@ -187,7 +221,7 @@ __device__ __forceinline__ void issue_rho(const StepArgs &a, const TileAdjArgs &
 }
 
 // CTAS as in tile.cuh
-template <bool MRT, int CTAS>
+template <bool MRT, int CTAS, bool WIDE>
 __global__ void __launch_bounds__(kTileThreads, CTAS)
     tile_adj_kernel(const StepArgs a, const AdjArgs d, const TileAdjArgs w) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -240,8 +274,12 @@ __global__ void __launch_bounds__(kTileThreads, CTAS)
             e = make_float2(a.eta2[r + xa], a.eta2[r + xb]);
         }
         sh.e2[v * kRows + j][T.lane] = e;
-        sh.sum[0][v * kRows + j][T.lane] = f2(0.f);
-        sh.sum[1][v * kRows + j][T.lane] = f2(0.f);
+        if (WIDE) {
+            sh.wide[v * kRows + j][T.lane] = make_double2(0., 0.);
+        } else {
+            sh.sum[0][v * kRows + j][T.lane] = f2(0.f);
+            sh.sum[1][v * kRows + j][T.lane] = f2(0.f);
+        }
     }
     // whether the region meets the sponge or a zero-ghost face, the source or receivers
     const int ylo = by * outy - K, sw = a.sponge_w;
@@ -285,11 +323,11 @@ __global__ void __launch_bounds__(kTileThreads, CTAS)
         const float2 above = v + 1 < kTileWarps ? sh.edge[par][v + 1 < kTileWarps ? v + 1 : v][1][T.lane]
                                                 : f2(0.f);
         if (special)  // warp-uniform
-            level<MRT, kSpecial>(a, d, w, T, sh, h, up, above, y0, l, own_rows, src_rows, rec_rows);
+            level<MRT, kSpecial, WIDE>(a, d, w, T, sh, h, up, above, y0, l, own_rows, src_rows, rec_rows);
         else if (gen)
-            level<MRT, kEdge>(a, d, w, T, sh, h, up, above, y0, l, own_rows, 0u, 0u);
+            level<MRT, kEdge, WIDE>(a, d, w, T, sh, h, up, above, y0, l, own_rows, 0u, 0u);
         else
-            level<MRT, kPlain>(a, d, w, T, sh, h, up, above, y0, l, own_rows, 0u, 0u);
+            level<MRT, kPlain, WIDE>(a, d, w, T, sh, h, up, above, y0, l, own_rows, 0u, 0u);
         if (l + 1 < K) issue_rho(a, w, T, sh, y0, l + 1, own_rows);
     }
     if (T.own) {
@@ -303,10 +341,16 @@ __global__ void __launch_bounds__(kTileThreads, CTAS)
                 if (pad) h[j][i].y = 0.f;
                 Two<float>::store(d.lam_out + Lat<5>::opp(i) * a.plane + o, h[j][i]);
             }
-            const float2 s0 = sh.sum[0][v * kRows + j][T.lane], s1 = sh.sum[1][v * kRows + j][T.lane];
+            double2 s;
+            if (WIDE) {
+                s = sh.wide[v * kRows + j][T.lane];
+            } else {
+                const float2 s0 = sh.sum[0][v * kRows + j][T.lane], s1 = sh.sum[1][v * kRows + j][T.lane];
+                s = make_double2((double)s0.x + (double)s1.x, (double)s0.y + (double)s1.y);
+            }
             double2 g = *reinterpret_cast<const double2 *>(d.grad + o);
-            g.x += (double)s0.x + (double)s1.x;
-            if (!pad) g.y += (double)s0.y + (double)s1.y;
+            g.x += s.x;
+            if (!pad) g.y += s.y;
             *reinterpret_cast<double2 *>(d.grad + o) = g;
         }
     }
@@ -317,21 +361,18 @@ __global__ void __launch_bounds__(kTileThreads, CTAS)
 using namespace lbtileadj;
 using namespace lbrt;
 
-// Levels of the next launch of n wanted ones (0: the wavefront's).  The cost of a tile as in
-// wave.cu's tile_cost; K evened out over the launches.
+// Levels of the next launch of n wanted ones (0: the wavefront's): 4 or 8, as costs less a level
+// (a tile's cost as in wave.cu's tile_cost), and what is left of four in FP64.
 int tile_adj_levels(const lb_ctx *ctx, int n) {
     if ((long long)ctx->ny * ctx->pitch >= 3500000) return 0;
-    int best = 2;
-    long long cost = -1;
-    for (int K = 2; K <= kLevels; K += 2) {
+    if (n < 4) return n;
+    auto cost = [&](int K) {
         const int ox = kSide - 2 * halo_x(K), oy = kSide - 2 * K;
         const long long t = (long long)((ctx->nx + ox - 1) / ox) * ((ctx->ny + oy - 1) / oy);
-        const long long c = t <= sm_count() ? 520 + 54 * K
-                                            : std::max<long long>(600 + 135 * K, 400 + t * (250 + 62 * K) / sm_count());
-        if (cost < 0 || c * best < cost * K) cost = c, best = K;
-    }
-    const int launches = (n + best - 1) / best;
-    return (n + launches - 1) / launches;
+        return t <= sm_count() ? 520 + 54 * K
+                               : std::max<long long>(600 + 135 * K, 400 + t * (250 + 62 * K) / sm_count());
+    };
+    return n >= kLevels && cost(kLevels) <= 2 * cost(4) ? kLevels : 4;
 }
 
 cudaError_t tile_adj_launch(lb_ctx *ctx, const StepArgs &a, const AdjArgs &d, const float *rho_hi,
@@ -349,9 +390,13 @@ cudaError_t tile_adj_launch(lb_ctx *ctx, const StepArgs &a, const AdjArgs &d, co
     w.tx = (ctx->nx + ox - 1) / ox;
     const int tiles = w.tx * ((ctx->ny + oy - 1) / oy);
     const bool mrt = ctx->cfg.collision == LB_MRT, one = tiles <= sm_count();
-    void (*fn)(const StepArgs, const AdjArgs, const TileAdjArgs) =
-        mrt ? (one ? tile_adj_kernel<true, 1> : tile_adj_kernel<true, 2>)
-            : (one ? tile_adj_kernel<false, 1> : tile_adj_kernel<false, 2>);
+    void (*fn)(const StepArgs, const AdjArgs, const TileAdjArgs);
+    if (K < 4)
+        fn = mrt ? (one ? tile_adj_kernel<true, 1, true> : tile_adj_kernel<true, 2, true>)
+                 : (one ? tile_adj_kernel<false, 1, true> : tile_adj_kernel<false, 2, true>);
+    else
+        fn = mrt ? (one ? tile_adj_kernel<true, 1, false> : tile_adj_kernel<true, 2, false>)
+                 : (one ? tile_adj_kernel<false, 1, false> : tile_adj_kernel<false, 2, false>);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(SharedAdj));
     if (e != cudaSuccess) return e;
