@@ -287,8 +287,9 @@ lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *grad_c, doub
  * records the forward rho tape or keeps checkpoints during its forward run
  * (lb_request.checkpoint_every) and its adjoint (lb_adjoint, J = 1/2
  * sum (p - d)^2 over its traces) runs on a worker thread on its own stream,
- * overlapping the batched forward work.  Results do not depend on what else
- * is in the batch: each shot runs the same kernels with the same arithmetic.
+ * overlapping the batched forward work.  Each shot runs the same kernels with
+ * the same arithmetic whatever else is in the batch, except for the rounding of
+ * BF16 shots (tb_min_ctas).
  */
 typedef struct lb_server lb_server;
 
@@ -297,13 +298,15 @@ typedef struct {
     size_t hbm_budget;       /* device bytes the server may hold; 0: 80% of free memory */
     int rounds_per_pass;     /* steps per scheduling pass between admission checks, >= 1 */
     int adjoint_workers;     /* threads running gradient sweeps, >= 1 */
-    int tb_min_ctas;         /* D2Q5 shots (FP32 with no checkpoint; BF16 also with no tape) can
-                                advance 4 steps per launch.  0: they do.  > 0: they do, at
-                                64 rows per warp, when together they make at least this many
-                                CTAs.  < 0: never.  FP32 results are the same bit for bit; so
-                                are BF16 results, except that BF16 shots keep FP32 between the
-                                4 steps of a launch with tb_min_ctas > 0, or with 0 while the
-                                ready shots together outgrow three quarters of L2. */
+    int tb_min_ctas;         /* D2Q5 FP32 and BF16 shots without checkpoints can advance 4 steps
+                                per launch.  0: they do.  > 0: they do, at 64 rows per warp,
+                                when together they make at least this many CTAs.  < 0: never.
+                                FP32 results are the same bit for bit, and so are those of BF16
+                                shots with a rho tape.  BF16 shots without one keep FP32 between
+                                the 4 steps of a launch when the ready shots without a tape
+                                make tb_min_ctas > 0 CTAs or, with 0, when their rows (of 248
+                                columns) are more than 33 per SM and their states outgrow
+                                three quarters of L2; they round at every step otherwise. */
 } lb_server_config;
 
 typedef struct {
