@@ -490,7 +490,8 @@ lb_status lb_footprint(const lb_config *cfg, int nt, int nrec, int want_adjoint,
     size_t b = nbuf * q * plane * elem_bytes(cfg->storage) + plane * 4 + plane + 1024;
     if (cfg->storage == LB_F64) b += plane * 8 + (size_t)std::max(nt, 0) * 8 + 256;
     if (nrec > 0 && nt > 0)
-        b += (size_t)nt * nrec * 4 + (size_t)nrec * 16 + (size_t)std::max(cfg->ny, 1) * 4 + 256;
+        b += (size_t)nt * nrec * 4 + (size_t)nrec * 20 + (size_t)std::max(cfg->ny, 1) * 4 + 512;
+    if (cfg->storage == LB_F16) b += kScaleSlots * 9 * (kMaxCopies + 1) * 4 + 256;  // range scales
     if (nt > 0) b += (size_t)nt * 4;
     // refinement levels (refine.cu): per patch, two population buffers with a ghost ring and
     // its eta^2 plane, the interface lists and three snapshot slots, the nested patch's
