@@ -202,9 +202,21 @@ __device__ __forceinline__ void tile_body(const StepArgs &a, const TileArgs &w, 
         }
         sh.med[v * kRows + j][T.lane] = make_float2(med_of<5>(m[j].x), med_of<5>(m[j].y));
     }
+    // a zero-ghost face among the warp's rows and columns: cut (wave.cuh: cut_left)
+    const bool face = !T.per && (x0 <= 0 || x0 + kSide >= a.nx - 1 || (y0 <= 0 && y0 + kRows > 0) ||
+                                 (y0 < a.ny && y0 + kRows >= a.ny));
 #pragma unroll 1
     for (int l = 0; l < K; l++) {
         const int par = l & 1;
+        if (face) {  // warp-uniform
+#pragma unroll
+            for (int j = 0; j < kRows; j++) {
+                cut_right(h[j][1], T.gx, a.nx);
+                cut_left(h[j][3], T.gx);
+                h[j][2] = y0 + j == a.ny - 1 ? f2(0.f) : h[j][2];
+                h[j][4] = y0 + j == 0 ? f2(0.f) : h[j][4];
+            }
+        }
         sh.edge[par][v][0][T.lane] = h[kRows - 1][2];
         sh.edge[par][v][1][T.lane] = h[0][4];
         __syncthreads();  // (by parity: the next step's edges overwrite those of the step before)

@@ -62,11 +62,16 @@ WavePick pick(const lb_ctx *c, int K, bool rec) {
     return c->cfg.storage == LB_BF16 ? pick_d2q5_bf16(ck, K, rec) : pick_d2q5_f32(ck, K, rec);
 }
 
-// What a row in the sponge counts against kInner: an iteration with sponge factors issues half as
-// many instructions again.  The four-step FP32 BGK launch waits for HBM in part and hides some
-// of that: 4/3 there (4096^2: 514 GLUPS against 496), 3/2 elsewhere (MRT: 525 against 451, six
-// steps: 570 against 546).
+// What a row in the sponge or of a strip at a face counts against kInner: an iteration with sponge
+// factors issues half as many instructions again, one with the cuts at a zero-ghost face (wave.cuh)
+// about as many again.  us a step at weights of 8 / 9 / 12 / 13 / 14 sixths, two-layer 4096^2 with a
+// sponge: BGK FP32 36.7 / 33.6 / 30.1 / 29.8 / 31.3, MRT 38.4 / 35.9 / 34.0 / 33.7 / 33.0, BF16 33.9 /
+// 33.6 / 33.6 / 32.8 / 32.3, D2Q9 MRT 83.5 / 77.6 / 70.8 / 69.7 / 69.9; without: 36.7 / 34.2 / 27.4 /
+// 27.3 / 27.3, 38.1 / 36.0 / 32.7 / 33.2 / 33.1, 32.1 / 29.6 / 28.8 / 29.7 / 29.7, 84.8 / 78.0 / 62.9 /
+// 65.1 / 65.3.  Periodic grids cut nothing: 4/3 where the four-step FP32 BGK launch waits for HBM in
+// part, 3/2 elsewhere.
 int outer_weight(const lb_ctx *c, int K) {
+    if (c->cfg.boundary != LB_PERIODIC) return c->cfg.sponge_width > 0 ? 13 : 12;
     return c->Q == 5 && K <= 4 && c->cfg.storage == LB_F32 && c->cfg.collision == LB_BGK ? 8 : 9;
 }
 

@@ -217,6 +217,15 @@ template <int Q> struct Range<Q, __half> {
     }
 };
 
+// Nothing crosses a face of a zero-ghost grid.  Sites beyond it are computed too and multiplied by 0,
+// but that keeps a non-finite value, which the one-step kernels lose across the face.  So what
+// leaves the first column to the left and the last to the right is set to 0.
+__device__ __forceinline__ void cut_left(float2 &h, int gx) { h.x = gx == 0 ? 0.f : h.x; }
+__device__ __forceinline__ void cut_right(float2 &h, int gx, int nx) {
+    h.x = gx == nx - 1 ? 0.f : h.x;
+    h.y = gx == nx - 2 ? 0.f : h.y;
+}
+
 // the values at x - 1 and x + 1 of a lane's columns
 __device__ __forceinline__ float2 from_left(float2 h) {
     return make_float2(__shfl_up_sync(0xffffffffu, h.y, 1), h.x);
@@ -327,6 +336,7 @@ struct Lane {
     bool live;             // zero ghost: some column inside the grid
     bool split;            // periodic: the two columns are not one aligned vector in memory
     bool src;              // warp-uniform: the source column is among the strip's
+    bool face;             // warp-uniform: so is a column next to a zero-ghost face
     unsigned src_cols;     // bit j: column j is the source's
     int rec_lo, rec_hi;    // first and last row of the chunk's receivers in this strip (none: 1, 0)
     bool dense;            // warp-uniform: more than 32 of them; otherwise one per lane:
@@ -592,6 +602,24 @@ __device__ __forceinline__ void iterate(const StepArgs &a, const WaveArgs &w, co
     at.in += a.pitch;
     at.mid += a.pitch;
     at.eta2 += a.pitch;
+    // Cuts at zero-ghost faces (cut_left), in one place ahead of the levels, which are short of
+    // registers and instruction fetch (two-layer 4096^2, 200 steps: 8390 us with the cuts in each
+    // level, 10530 with levels of their own for the warps at a face, 7410 here and 6690 once those
+    // warps' rows count more, outer_weight; 6840 without cuts and at the rows' old weight)
+    if (!FAST && !T.per && (T.face || r <= K || r >= a.ny)) {  // warp-uniform
+#pragma unroll
+        for (int l = 0; l < K; l++) {
+            cut_right(S.z[l][1], T.gx, a.nx);
+            cut_left(S.z[l][2], T.gx);
+            const bool row = r - l - 1 < 1 || r - l - 1 >= a.ny;  // of the rows -1 and ny - 1
+#pragma unroll
+            for (int i = 0; i < Levels<Q, K>::NP; i++) S.p[P][l][i] = row ? f2(0.f) : S.p[P][l][i];
+            if constexpr (Q == 9) {
+                cut_right(S.p[P][l][1], T.gx, a.nx);
+                cut_left(S.p[P][l][2], T.gx);
+            }
+        }
+    }
 #pragma unroll
     for (int l = 0; l < K; l++) {
         const int y = r - l - 1;  // the row level l + 1 computes
@@ -614,6 +642,10 @@ __device__ __forceinline__ void iterate(const StepArgs &a, const WaveArgs &w, co
         S.z[l][2] = n[3];
         S.p[P][l][0] = n[2];
         if constexpr (Q == 9) {
+            if (!FAST && !T.per) {
+                cut_left(n[7], T.gx);
+                cut_right(n[8], T.gx, a.nx);
+            }
             g[5] = from_left(S.p[P][l][1]);
             g[6] = from_right(S.p[P][l][2]);
             g[7] = from_right(n[7]);
@@ -717,6 +749,7 @@ __device__ __forceinline__ void sweep(const StepArgs &a, const WaveArgs &w, int 
         if (x == a.src_x) T.src_cols |= 1u << j;
     }
     T.fx = make_float2(f[0], f[1]);
+    T.face = __any_sync(0xffffffffu, !T.per && (T.gx == 0 || T.gx == a.nx - 1 || T.gx == a.nx - 2));
     T.src = __any_sync(0xffffffffu, T.src_cols != 0) && a.src_tab != nullptr && a.t < a.src_nt;
     if (work) find_receivers(w, T, T.med - T.lane * 16);
     cp_wait<kRing - 1>();  // the table (its group came first)
@@ -731,7 +764,7 @@ __device__ __forceinline__ void sweep(const StepArgs &a, const WaveArgs &w, int 
         for (int i = 0; i < Levels<Q, K>::NP; i++) S.p[0][l][i] = S.p[1][l][i] = f2(0.f);
     }
     // FAST iterations: [f0, f1) without those that meet the source or receiver rows
-    int f0 = max(T.Y0, a.sponge_w) + K;
+    int f0 = max(T.Y0, max(a.sponge_w, T.per ? 0 : 1)) + K;  // (1: nothing to cut)
     // (the row that an iteration takes in counts too: its sponge factor is noted as 1)
     int f1 = min(min(T.Y1 + 1, rend - kRing + 1), min(a.ny - a.sponge_w, a.ny - kRing + 1));
     if (__any_sync(0xffffffffu, xedge || T.split || (T.own && T.gx + 1 >= a.nx))) f1 = f0;
