@@ -242,7 +242,11 @@ Fuse fuse_steps(const lb_ctx *c, int n) {
     // a second launch that mostly ends at once; 3001 x 1777: 25.5 us a step against 35.9).  They pay
     // against the staged step (1420 x 675: 12.1 against 17.0), not against the register-streaming one
     // of narrower grids (431 x 1307: 11.4 against 9.1).
-    if (c->cfg.storage == LB_F16) return Fuse{n >= 2 && c->staged && sites >= 500000 ? 2 : 1, false};
+    // At the seam of odd periodic rows a 16-bit wavefront copies value by value, while the other strips
+    // wait (FP16 1471 x 3767: 57 us a step against 38; BF16 4017 x 3861: 88 against 63).
+    const bool seam = c->cfg.boundary == LB_PERIODIC && c->nx % 2 != 0;
+    if (c->cfg.storage == LB_F16)
+        return Fuse{n >= 2 && c->staged && sites >= 500000 && !seam ? 2 : 1, false};
     if (c->Q == 5 && sites < 3500000) {
         if (n < 2) return Fuse{1, false};
         int best = 2;
@@ -255,15 +259,12 @@ Fuse fuse_steps(const lb_ctx *c, int n) {
         if (tile_cost(c, K) >= K * (310 + sites * 6 / 10000)) return Fuse{1, false};
         return Fuse{K, true};
     }
+    if (seam && c->cfg.storage == LB_BF16) return Fuse{1, false};
     if (c->cfg.time_block <= 1) {
         if (!wave_pays(c)) return Fuse{1, false};
         // D2Q9 FP32 grids below a million sites run one step as fast in L2 (708 x 739 MRT: 8.7 us
-        // against 9.9, 374 x 3184: 16.6 against 13.9); BF16 rows of odd periodic grids come value by
-        // value at the seam, while the other strips wait (1443 x 1358: 27.5 against 37.0)
-        if (c->Q == 9 && (c->cfg.storage == LB_BF16
-                              ? c->cfg.boundary == LB_PERIODIC && c->nx % 2 != 0
-                              : sites < 1000000))
-            return Fuse{1, false};
+        // against 9.9, 374 x 3184: 16.6 against 13.9)
+        if (c->Q == 9 && c->cfg.storage == LB_F32 && sites < 1000000) return Fuse{1, false};
     }
     return Fuse{wave_steps(c, n), false};
 }
