@@ -16,6 +16,48 @@ bool sweep3_supported(const lb_ctx *c) {
            (c->cfg.storage == LB_F32 || c->cfg.storage == LB_BF16);
 }
 
+namespace {
+
+// Tiles and chunks of a launch, and about what it takes: `rounds` planes one after another, of which a
+// CTA computes `rows` rows each.
+struct Plan {
+    SweepArgs w;
+    long long rounds;
+    int rows;
+    bool one_wave;
+};
+
+Plan plan_of(const lb_ctx *ctx) {
+    Plan p;
+    SweepArgs &w = p.w;
+    w.per = ctx->cfg.boundary == LB_PERIODIC ? 1 : 0;
+    w.rec_blocks = 0;
+    // tiles evened out; their sides multiples of 8 columns (whole 32-byte sectors in FP32) where
+    // one tile does not take the row
+    const int most = kMaxX / 8 * 8;
+    w.tx = ctx->nx <= kMaxX ? 1 : (ctx->nx + most - 1) / most;
+    w.outx = round_up((ctx->nx + w.tx - 1) / w.tx, w.tx == 1 ? 2 : 8);
+    w.ty = (ctx->ny3 + kMaxY - 1) / kMaxY;
+    w.outy = (ctx->ny3 + w.ty - 1) / w.ty;
+    // chunks of planes: a CTA takes its planes and two more, and about two planes' time to start;
+    // two CTAs share an SM.  The receivers' blocks, which come first, are short: they count nothing here
+    // (256^3 with 160000 receivers: 143 us a step, 468 when they were taken off the slots)
+    const long long tiles = (long long)w.tx * w.ty, slots = 2 * sm_count();
+    p.rounds = -1;
+    w.chunks = 1;
+    for (int n = 1; n <= ctx->nz; n++) {
+        const long long waves = (tiles * n + slots - 1) / slots;
+        const long long c = waves * ((ctx->nz + n - 1) / n + 4);
+        if (p.rounds < 0 || c < p.rounds) p.rounds = c, w.chunks = n;
+        if (waves > 4) break;
+    }
+    p.rows = std::min(w.outy + 2 * kHaloY, kRegY);
+    p.one_wave = tiles * w.chunks <= slots;
+    return p;
+}
+
+}  // namespace
+
 // Where both states stay in L2 the one-step kernels are as fast or faster (us a step, one / two per
 // launch: FP32 96^3 10.2 / 11.5, 128^3 20.2 / 21.5, 192^3 74.8 / 55.4, 320^3 309 / 212; BF16, whose
 // one-step kernel converts twice as often: 64^3 8.5 / 8.7, 96^3 15.0 / 11.9, 128^3 24.6 / 21.0; staged
@@ -29,34 +71,15 @@ bool sweep3_pays(const lb_ctx *c) {
 // Two steps with the caller's arguments (a.in must not be raw); the receivers' two rows when
 // a.trace_row is set.
 lb_status sweep3_launch(lb_ctx *ctx, const StepArgs &a) {
-    SweepArgs w;
-    w.per = ctx->cfg.boundary == LB_PERIODIC ? 1 : 0;
+    SweepArgs w = plan_of(ctx).w;
     w.rec_blocks = a.trace_row ? (ctx->nrec + kThreadsZ - 1) / kThreadsZ : 0;
-    // tiles evened out; their sides multiples of 8 columns (whole 32-byte sectors in FP32) where
-    // one tile does not take the row
-    const int most = kMaxX / 8 * 8;
-    w.tx = ctx->nx <= kMaxX ? 1 : (ctx->nx + most - 1) / most;
-    w.outx = round_up((ctx->nx + w.tx - 1) / w.tx, w.tx == 1 ? 2 : 8);
-    w.ty = (ctx->ny3 + kMaxY - 1) / kMaxY;
-    w.outy = (ctx->ny3 + w.ty - 1) / w.ty;
-    // chunks of planes: a CTA takes its planes and two more, and about two planes' time to start;
-    // two CTAs share an SM
-    const int sms = sm_count(), tiles = w.tx * w.ty, slots = std::max(1, 2 * sms - w.rec_blocks);
-    long long cost = -1;
-    w.chunks = 1;
-    for (int n = 1; n <= ctx->nz; n++) {
-        const long long waves = ((long long)tiles * n + slots - 1) / slots;
-        const long long c = waves * ((ctx->nz + n - 1) / n + 4);
-        if (cost < 0 || c < cost) cost = c, w.chunks = n;
-        if (waves > 4) break;
-    }
     const bool bf = ctx->cfg.storage == LB_BF16;
     const int smem = bf ? (int)sizeof(SharedZ<__nv_bfloat16>) : (int)sizeof(SharedZ<float>);
     void (*fn)(const StepArgs, const SweepArgs) =
         bf ? sweep3_kernel<__nv_bfloat16> : sweep3_kernel<float>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
-        e = launch_pdl(fn, dim3(w.rec_blocks + tiles * w.chunks), dim3(kThreadsZ), smem, ctx->stream,
+        e = launch_pdl(fn, dim3(w.rec_blocks + w.tx * w.ty * w.chunks), dim3(kThreadsZ), smem, ctx->stream,
                        a, w);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "3-D sweep launch");
     return LB_OK;
