@@ -59,13 +59,36 @@ Plan plan_of(const lb_ctx *ctx) {
 }  // namespace
 
 // Where both states stay in L2 the one-step kernels are as fast or faster (us a step, one / two per
-// launch: FP32 96^3 10.2 / 11.5, 128^3 20.2 / 21.5, 192^3 74.8 / 55.4, 320^3 309 / 212; BF16, whose
-// one-step kernel converts twice as often: 64^3 8.5 / 8.7, 96^3 15.0 / 11.9, 128^3 24.6 / 21.0; staged
-// (1100 x 40 x 40) 13.3 / 15.7, 320^3 290 / 162).  Odd periodic grids, whose rows are not whole
-// lanes at the seam, keep single steps too.
+// launch: FP32 96^3 10.4 / 11.5, 128^3 20.2 / 21.5, 192^3 74.8 / 55.4, 320^3 309 / 212; staged BF16
+// 1100 x 40 x 40 13.3 / 15.7, 320^3 290 / 162), so FP32 and staged grids have a line in sites.  Odd
+// periodic grids, whose rows are not whole lanes at the seam, keep single steps.
+//
+// Otherwise the estimates below decide, in us: a step of the one-step kernel by the warps' segments of a
+// row (128 sites, BF16 256) that it reads, filled or not, and a launch of two by its rounds of planes,
+// their rows and the receivers, whose second pressure costs 49 loads.  They are fits to 110 grids of
+// 0.2 to 17 million sites, good to 15 %; what they decide, us a step, one / two per launch: BF16 96^3
+// 12.7 / 12.2, periodic 12.6 / 14.8; 112 x 294 x 301 131 / 57; 238 x 68 x 129 15.2 / 20.2;
+// 208 x 227 x 82 29.5 / 28.2, periodic 28.0 / 34.9; 256^3 107 / 109, with 60000 receivers 108 / 117; FP32
+// periodic 184 x 254 x 62 31.5 / 33.5; 96 x 269 x 126 34.4 / 34.3.  Several waves of CTAs overlap, and
+// the estimate of a launch does not hold for them: they stay with the line in sites.
 bool sweep3_pays(const lb_ctx *c) {
-    if (c->cfg.boundary == LB_PERIODIC && c->nx % 2 != 0) return false;
-    return (long long)c->ny * c->pitch >= (c->cfg.storage == LB_BF16 && !c->staged ? 800000 : 3000000);
+    const bool per = c->cfg.boundary == LB_PERIODIC, bf = c->cfg.storage == LB_BF16;
+    if (per && c->nx % 2 != 0) return false;
+    if ((long long)c->ny * c->pitch < (bf && !c->staged ? 800000 : 3000000)) return false;
+    if (c->staged) return true;
+    const Plan p = plan_of(c);
+    if (!p.one_wave) return true;
+    const int seg = bf ? 256 : 128;
+    const double sites = 1e-6 * c->nx * c->ny, read = 1e-6 * round_up(c->nx, seg) * c->ny;
+    double one, round;  // a step; a round of planes
+    if (bf) {
+        one = 0.97 * (2.5 + (per ? 3.6 : 4.0) * read + 2.4 * sites);
+        round = per ? 1.2 + 0.125 * p.rows : 0.9 + 0.113 * p.rows;
+    } else {
+        one = std::max(8.0 * read, 9.8 * sites);
+        round = per ? 0.7 + 0.155 * p.rows : 0.4 + 0.135 * p.rows;
+    }
+    return p.rounds * round + 0.45e-3 * c->nrec < 2 * one;
 }
 
 // Two steps with the caller's arguments (a.in must not be raw); the receivers' two rows when

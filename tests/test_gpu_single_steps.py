@@ -73,7 +73,7 @@ def test_many_receivers_leave_the_sweep_its_ctas(sim_cls):
 # and those of both steps are recorded, in more blocks than the sweep has slots
 def test_many_receivers_are_recorded(sim_cls):
     import torch
-    nx, ny, nz, nrec, steps = 96, 181, 200, 170000, 5
+    nx, ny, nz, nrec, steps = 256, 250, 256, 170000, 5
     rng = np.random.default_rng(2)
     rec = np.stack([rng.integers(0, n, nrec) for n in (nx, ny, nz)], 1)
     g0, out = torch.randn(7, nz, ny, nx, device="cuda"), []
@@ -82,7 +82,23 @@ def test_many_receivers_are_recorded(sim_cls):
                       step_kernel=how)
         sim.set_receivers(rec, steps)
         sim.set_state(g0)
+        before = sim.info()[6]
         sim.step(steps)
+        assert sim.info()[6] - before == (steps if how == "direct" else 3)
         out.append(sim.traces(steps).clone())
         sim.close()
     assert torch.equal(out[0], out[1])
+
+
+# flat and periodic D3Q7 grids, and many receivers on small ones
+@pytest.mark.parametrize("storage,nx,ny,nz,boundary,nrec,launches", [
+    ("bf16", 238, 68, 129, "zero", 10, 8), ("bf16", 208, 139, 74, "periodic", 10, 8),
+    ("bf16", 208, 227, 82, "periodic", 10, 8), ("bf16", 192, 103, 417, "periodic", 10, 8),
+    ("bf16", 128, 128, 128, "periodic", 10, 8), ("f32", 184, 254, 62, "periodic", 10, 8),
+    ("bf16", 256, 256, 256, "zero", 60000, 8), ("f32", 135, 229, 106, "zero", 100000, 8),
+    ("bf16", 96, 96, 96, "zero", 10, 4), ("bf16", 112, 294, 301, "zero", 10, 4),
+    ("bf16", 164, 211, 179, "periodic", 10, 4), ("f32", 135, 229, 106, "zero", 1000, 4),
+    ("f32", 256, 256, 256, "zero", 160000, 4)])
+def test_d3q7_shapes(sim_cls, storage, nx, ny, nz, boundary, nrec, launches):
+    assert _launches(sim_cls, (nz, ny, nx), [8], nrec, lattice=7, storage=storage,
+                     boundary=boundary) == launches
