@@ -263,8 +263,13 @@ Fuse fuse_steps(const lb_ctx *c, int n) {
     if (c->cfg.time_block <= 1) {
         if (!wave_pays(c)) return Fuse{1, false};
         // D2Q9 FP32 grids below a million sites run one step as fast in L2 (708 x 739 MRT: 8.7 us
-        // against 9.9, 374 x 3184: 16.6 against 13.9)
-        if (c->Q == 9 && c->cfg.storage == LB_F32 && sites < 1000000) return Fuse{1, false};
+        // against 9.9, 374 x 3184: 16.6 against 13.9), odd periodic ones below two (297 x 4006: 15.2
+        // against 16.2, 1183 x 1183 in threes 15.9 against 17.2; 1415 x 1413: 25.8 against 20.4)
+        if (c->Q == 9 && c->cfg.storage == LB_F32 && sites < (seam ? 1800000 : 1000000))
+            return Fuse{1, false};
+        // two steps at a time: odd periodic D2Q5 grids of less than 5.4 million sites (1923 x 1924: 23.7
+        // against 25.0, 2345 x 2345: 35.3 against 32.9)
+        if (c->Q == 5 && seam && n < 4 && sites < 5400000) return Fuse{1, false};
     }
     return Fuse{wave_steps(c, n), false};
 }

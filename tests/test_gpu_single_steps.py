@@ -102,3 +102,13 @@ def test_many_receivers_are_recorded(sim_cls):
 def test_d3q7_shapes(sim_cls, storage, nx, ny, nz, boundary, nrec, launches):
     assert _launches(sim_cls, (nz, ny, nx), [8], nrec, lattice=7, storage=storage,
                      boundary=boundary) == launches
+
+
+# odd periodic FP32 rows: the seam costs less there, but not nothing
+@pytest.mark.parametrize("lattice,nx,ny,boundary,calls,launches", [
+    (9, 297, 4006, "periodic", [8], 8), (9, 1183, 1183, "periodic", [8], 8),
+    (9, 1415, 1413, "periodic", [8], 2), (9, 1184, 1183, "periodic", [8], 2), (9, 1183, 1183, "zero", [8], 2),
+    (5, 1923, 1924, "periodic", [2, 3], 5), (5, 1923, 1924, "periodic", [8], 2),
+    (5, 1924, 1924, "periodic", [2, 3], 3), (5, 2345, 2345, "periodic", [2, 3], 3)])
+def test_seam_of_odd_fp32_rows(sim_cls, lattice, nx, ny, boundary, calls, launches):
+    assert _launches(sim_cls, (ny, nx), calls, lattice=lattice, tau=0.6, boundary=boundary) == launches
