@@ -248,7 +248,9 @@ Fuse fuse_steps(const lb_ctx *c, int n) {
     if (c->cfg.storage == LB_F16)
         return Fuse{n >= 2 && c->staged && sites >= 500000 && !seam ? 2 : 1, false};
     if (c->Q == 5 && sites < 3500000) {
-        if (n < 2) return Fuse{1, false};
+        // two steps alone: a launch of tiles takes 8 us however few they are (614 x 117 periodic: 4.2 us a
+        // step against 2.9, 991 x 996: 6.0 against 5.4; three: 2.9 against 2.9)
+        if (n < 2 || (n == 2 && c->cfg.time_block <= 1)) return Fuse{1, false};
         int best = 2;
         long long cost = -1;
         for (int K = 2; K <= 16; K += 2) {

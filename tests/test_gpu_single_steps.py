@@ -112,3 +112,11 @@ def test_d3q7_shapes(sim_cls, storage, nx, ny, nz, boundary, nrec, launches):
     (5, 1924, 1924, "periodic", [2, 3], 3), (5, 2345, 2345, "periodic", [2, 3], 3)])
 def test_seam_of_odd_fp32_rows(sim_cls, lattice, nx, ny, boundary, calls, launches):
     assert _launches(sim_cls, (ny, nx), calls, lattice=lattice, tau=0.6, boundary=boundary) == launches
+
+
+# D2Q5 grids on tiles: two steps alone do not pay for a launch of tiles
+@pytest.mark.parametrize("storage,nx,ny", [("f32", 614, 117), ("bf16", 991, 996), ("f32", 1900, 557)])
+def test_two_steps_of_a_small_grid(sim_cls, storage, nx, ny):
+    kw = dict(storage=storage, boundary="periodic", collision="bgk")
+    assert _launches(sim_cls, (ny, nx), [2, 2, 1], **kw) == 5
+    assert _launches(sim_cls, (ny, nx), [3, 8], **kw) == 2
