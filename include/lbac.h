@@ -288,8 +288,8 @@ lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *grad_c, doub
  * (lb_request.checkpoint_every) and its adjoint (lb_adjoint, J = 1/2
  * sum (p - d)^2 over its traces) runs on a worker thread on its own stream,
  * overlapping the batched forward work.  Each shot runs the same kernels with
- * the same arithmetic whatever else is in the batch, except for the rounding of
- * BF16 shots (tb_min_ctas).
+ * the same arithmetic whatever else is in the batch, except that what else there
+ * is decides how often BF16 shots round (tb_min_ctas).
  */
 typedef struct lb_server lb_server;
 
@@ -302,9 +302,9 @@ typedef struct {
                                 per launch.  0: they do.  > 0: they do, at 64 rows per warp,
                                 when together they make at least this many CTAs.  < 0: never.
                                 FP32 results are the same bit for bit, and so are those of BF16
-                                shots with a rho tape.  BF16 shots without one keep FP32 between
-                                the 4 steps of a launch when the ready shots without a tape
-                                make tb_min_ctas > 0 CTAs or, with 0, when their rows (of 248
+                                shots with a rho tape, which round at every step.  BF16 shots
+                                without one keep FP32 between the 4 steps of a launch with
+                                tb_min_ctas > 0, or with 0 while the ready shots' rows (of 248
                                 columns) are more than 33 per SM and their states outgrow
                                 three quarters of L2; they round at every step otherwise. */
 } lb_server_config;

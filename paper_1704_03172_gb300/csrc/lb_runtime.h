@@ -189,8 +189,7 @@ lb_status sweep3_launch(lb_ctx *ctx, const lbk::StepArgs &a);
 // together, a shot's CTAs at H rows per warp, the fill (advancing the shots) and the launch from
 // the device copy of the staging block.  BF16 shots round at every step, as the one-step
 // kernels do, while the shots in hand are few; once they fill a wave of 12 rows x 248 columns
-// per CTA slot and outgrow three quarters of L2 they keep FP32 between the steps of a launch.  Shots
-// with a rho tape do not count: their company leaves the others' results as they are.
+// per CTA slot and outgrow three quarters of L2 they keep FP32 between the steps of a launch.
 constexpr int kServeSteps = 4;
 size_t wave_batch_bytes(int n);
 bool wave_batch_ready(const lb_ctx *ctx);

@@ -378,14 +378,9 @@ void pass(lb_server *S) {
     if (!tbs.empty()) {
         bool use = true;
         if (S->cfg.tb_min_ctas > 0) {
-            long long ctas = 0, untaped = 0;
-            for (Req *r : tbs) {
-                const int n = wave_batch_blocks(r->ctx, tb_rows);
-                ctas += n;
-                if (!r->ctx->rho_tape) untaped += n;
-            }
+            long long ctas = 0;
+            for (Req *r : tbs) ctas += wave_batch_blocks(r->ctx, tb_rows);
             use = ctas >= S->cfg.tb_min_ctas;
-            round = untaped < S->cfg.tb_min_ctas;
         } else {
             for (Req *r : tbs) cs.push_back(r->ctx);
             tb_rows = wave_batch_rows(cs.data(), (int)cs.size());

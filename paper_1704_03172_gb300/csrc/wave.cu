@@ -393,7 +393,6 @@ bool wave_batch_round(lb_ctx *const *ctxs, int n) {
     }
     long long rows = 0, state = 0;
     for (int k = 0; k < n; k++) {
-        if (ctxs[k]->rho_tape) continue;
         rows += (long long)((ctxs[k]->nx + 247) / 248) * ctxs[k]->ny;
         state += 2LL * ctxs[k]->Q * ctxs[k]->ny * ctxs[k]->pitch * ctxs[k]->ebytes;
     }
