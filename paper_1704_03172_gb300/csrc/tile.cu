@@ -2,5 +2,5 @@
 #include "tile.cuh"
 
 namespace lbtile {
-TileFn pick_tile_f32(int ck, bool rec, int ctas) { return pick_tile<float>(ck, rec, ctas); }
+TileFn pick_tile_f32(int ck, bool rec, int ctas, bool per) { return pick_tile<float>(ck, rec, ctas, per); }
 }  // namespace lbtile

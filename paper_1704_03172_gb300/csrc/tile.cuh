@@ -97,13 +97,13 @@ __device__ __forceinline__ void tile_rows(const StepArgs &a, const TileArgs &w, 
     }
 }
 
-template <int CK, bool REC, typename ST>
+template <int CK, bool REC, typename ST, bool PER>
 __device__ __forceinline__ void tile_body(const StepArgs &a, const TileArgs &w, int tile, Shared &sh) {
     const int K = w.K, hx = halo_x(K), outx = kSide - 2 * hx, outy = kSide - 2 * K;
     const int by = tile / w.tx, bx = tile - by * w.tx, v = threadIdx.x >> 5;
     Lane T;
     T.lane = threadIdx.x & 31;
-    T.per = w.rec.per != 0;
+    T.per = PER;
     const int x0 = bx * outx - hx, y0 = by * outy - K + v * kRows;  // the region's, the warp's first
     T.gx = x0 + 2 * T.lane;
     T.gxw = T.gx;
@@ -202,17 +202,23 @@ __device__ __forceinline__ void tile_body(const StepArgs &a, const TileArgs &w, 
         }
         sh.med[v * kRows + j][T.lane] = make_float2(med_of<5>(m[j].x), med_of<5>(m[j].y));
     }
-    // a zero-ghost face among the warp's rows and columns: cut (wave.cuh: cut_left)
-    const bool face = !T.per && (x0 <= 0 || x0 + kSide >= a.nx - 1 || (y0 <= 0 && y0 + kRows > 0) ||
-                                 (y0 < a.ny && y0 + kRows >= a.ny));
+    // zero-ghost faces among the warp's columns and rows: cut (wave.cuh: cut_left)
+    const bool left = !T.per && x0 <= 0, right = !T.per && x0 + kSide >= a.nx - 1,
+               rows = !T.per && ((y0 <= 0 && y0 + kRows > 0) || (y0 < a.ny && y0 + kRows >= a.ny));
 #pragma unroll 1
     for (int l = 0; l < K; l++) {
         const int par = l & 1;
-        if (face) {  // warp-uniform
+        if (left) {  // warp-uniform, as the next two
+#pragma unroll
+            for (int j = 0; j < kRows; j++) cut_left(h[j][3], T.gx);
+        }
+        if (right) {
+#pragma unroll
+            for (int j = 0; j < kRows; j++) cut_right(h[j][1], T.gx, a.nx);
+        }
+        if (rows) {
 #pragma unroll
             for (int j = 0; j < kRows; j++) {
-                cut_right(h[j][1], T.gx, a.nx);
-                cut_left(h[j][3], T.gx);
                 h[j][2] = y0 + j == a.ny - 1 ? f2(0.f) : h[j][2];
                 h[j][4] = y0 + j == 0 ? f2(0.f) : h[j][4];
             }
@@ -249,26 +255,29 @@ __device__ __forceinline__ void tile_body(const StepArgs &a, const TileArgs &w, 
 
 // CTAS: 1 (112 registers) where the tiles are no more than the SMs, else 2 per SM (64 registers,
 // with spills, and still faster: 1024^2 3.5 against 3.7 us a step, 2048^2 11.0 against 14.9)
-template <int CK, bool REC, typename ST, int CTAS>
+template <int CK, bool REC, typename ST, int CTAS, bool PER>
 __global__ void __launch_bounds__(kTileThreads, CTAS) tile_kernel(const StepArgs a, const TileArgs w) {
     extern __shared__ __align__(16) unsigned char smem[];
     Shared &sh = *reinterpret_cast<Shared *>(smem);
     asm volatile("griddepcontrol.wait;" ::: "memory");  // (no early launch of dependents: wave.cuh)
-    tile_body<CK, REC, ST>(a, w, blockIdx.x, sh);
+    tile_body<CK, REC, ST, PER>(a, w, blockIdx.x, sh);
 }
 
 using TileFn = void (*)(const StepArgs, const TileArgs);
 
-template <typename ST, int CTAS> TileFn pick_tile_c(int ck, bool rec) {
-    if (ck == kMrt) return rec ? tile_kernel<kMrt, true, ST, CTAS> : tile_kernel<kMrt, false, ST, CTAS>;
+template <typename ST, int CTAS, bool PER> TileFn pick_tile_c(int ck, bool rec) {
+    if (ck == kMrt)
+        return rec ? tile_kernel<kMrt, true, ST, CTAS, PER> : tile_kernel<kMrt, false, ST, CTAS, PER>;
     if (ck == kLossless)
-        return rec ? tile_kernel<kLossless, true, ST, CTAS> : tile_kernel<kLossless, false, ST, CTAS>;
-    return rec ? tile_kernel<kBgk, true, ST, CTAS> : tile_kernel<kBgk, false, ST, CTAS>;
+        return rec ? tile_kernel<kLossless, true, ST, CTAS, PER>
+                   : tile_kernel<kLossless, false, ST, CTAS, PER>;
+    return rec ? tile_kernel<kBgk, true, ST, CTAS, PER> : tile_kernel<kBgk, false, ST, CTAS, PER>;
 }
-template <typename ST> TileFn pick_tile(int ck, bool rec, int ctas) {
-    return ctas == 1 ? pick_tile_c<ST, 1>(ck, rec) : pick_tile_c<ST, 2>(ck, rec);
+template <typename ST> TileFn pick_tile(int ck, bool rec, int ctas, bool per) {
+    if (per) return ctas == 1 ? pick_tile_c<ST, 1, true>(ck, rec) : pick_tile_c<ST, 2, true>(ck, rec);
+    return ctas == 1 ? pick_tile_c<ST, 1, false>(ck, rec) : pick_tile_c<ST, 2, false>(ck, rec);
 }
-TileFn pick_tile_f32(int ck, bool rec, int ctas);   // tile.cu
-TileFn pick_tile_bf16(int ck, bool rec, int ctas);  // tile_bf16.cu
+TileFn pick_tile_f32(int ck, bool rec, int ctas, bool per);   // tile.cu
+TileFn pick_tile_bf16(int ck, bool rec, int ctas, bool per);  // tile_bf16.cu
 
 }  // namespace lbtile

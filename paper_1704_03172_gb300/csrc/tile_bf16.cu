@@ -2,5 +2,5 @@
 #include "tile.cuh"
 
 namespace lbtile {
-TileFn pick_tile_bf16(int ck, bool rec, int ctas) { return pick_tile<__nv_bfloat16>(ck, rec, ctas); }
+TileFn pick_tile_bf16(int ck, bool rec, int ctas, bool per) { return pick_tile<__nv_bfloat16>(ck, rec, ctas, per); }
 }  // namespace lbtile

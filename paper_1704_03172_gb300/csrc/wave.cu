@@ -18,13 +18,13 @@ using namespace lbwave;
 using namespace lbtile;
 
 namespace lbwave {
-WavePick pick_d2q5_f32(int ck, int K, bool rec) {
+WavePick pick_d2q5_f32(int ck, int K, bool rec, bool per) {
     if (K == 6)  // BGK only (wave_steps)
-        return ck == kLossless ? rec ? pick_one<5, kLossless, 6, true, float, false>()
-                                     : pick_one<5, kLossless, 6, false, float, false>()
-                               : rec ? pick_one<5, kBgk, 6, true, float, false>()
-                                     : pick_one<5, kBgk, 6, false, float, false>();
-    return K == 4 ? pick_rec<5, 4, float, false>(ck, rec) : pick_rec<5, 2, float, false>(ck, rec);
+        return ck == kLossless ? rec ? pick_one<5, kLossless, 6, true, float, false>(per)
+                                     : pick_one<5, kLossless, 6, false, float, false>(per)
+                               : rec ? pick_one<5, kBgk, 6, true, float, false>(per)
+                                     : pick_one<5, kBgk, 6, false, float, false>(per);
+    return K == 4 ? pick_rec<5, 4, float, false>(ck, rec, per) : pick_rec<5, 2, float, false>(ck, rec, per);
 }
 WaveBatchFn pick_batch_fp32(bool mrt) { return pick_batch<false>(mrt); }
 }  // namespace lbwave
@@ -56,22 +56,29 @@ int collision_kind(const lb_ctx *c) {
 
 WavePick pick(const lb_ctx *c, int K, bool rec) {
     const int ck = collision_kind(c);
+    const bool per = c->cfg.boundary == LB_PERIODIC;
     if (c->Q == 9)
-        return c->cfg.storage == LB_BF16 ? pick_d2q9_bf16(ck, K, rec) : pick_d2q9_f32(ck, K, rec);
-    if (c->cfg.storage == LB_F16) return pick_d2q5_f16(ck, rec);
-    return c->cfg.storage == LB_BF16 ? pick_d2q5_bf16(ck, K, rec) : pick_d2q5_f32(ck, K, rec);
+        return c->cfg.storage == LB_BF16 ? pick_d2q9_bf16(ck, K, rec, per)
+                                         : pick_d2q9_f32(ck, K, rec, per);
+    if (c->cfg.storage == LB_F16) return pick_d2q5_f16(ck, rec, per);
+    return c->cfg.storage == LB_BF16 ? pick_d2q5_bf16(ck, K, rec, per) : pick_d2q5_f32(ck, K, rec, per);
 }
 
 // What a row in the sponge or of a strip at a face counts against kInner: an iteration with sponge
 // factors issues half as many instructions again, one with the cuts at a zero-ghost face (wave.cuh)
-// about as many again.  us a step at weights of 8 / 9 / 12 / 13 / 14 sixths, two-layer 4096^2 with a
-// sponge: BGK FP32 36.7 / 33.6 / 30.1 / 29.8 / 31.3, MRT 38.4 / 35.9 / 34.0 / 33.7 / 33.0, BF16 33.9 /
-// 33.6 / 33.6 / 32.8 / 32.3, D2Q9 MRT 83.5 / 77.6 / 70.8 / 69.7 / 69.9; without: 36.7 / 34.2 / 27.4 /
-// 27.3 / 27.3, 38.1 / 36.0 / 32.7 / 33.2 / 33.1, 32.1 / 29.6 / 28.8 / 29.7 / 29.7, 84.8 / 78.0 / 62.9 /
-// 65.1 / 65.3.  Periodic grids cut nothing: 4/3 where the four-step FP32 BGK launch waits for HBM in
-// part, 3/2 elsewhere.
+// more.  Times of 85 zero-ghost grids of 0.2 to 25 million sites at weights of 8 / 9 / 10 / 11 / 12 / 13 / 14
+// sixths against the best: with a sponge D2Q5 FP32 1.06 / 1.03 / 1.01 / 1.01 / 1.01 / 1.00 / 1.00, BF16 1.06 /
+// 1.04 / 1.03 / 1.01 / 1.00 / 1.00 / 1.00, D2Q9 BF16 1.06 / 1.02 / 1.00 / 1.00 / 1.00 / 1.01 / 1.01, FP32
+// 1.12 / 1.08 / 1.03 / 1.01 / 1.00 / 1.00 / 1.00; without D2Q5 BF16 1.00 / 1.01 / 1.02 / 1.02 / 1.03 / 1.04 / 1.03,
+// the others about as with; six steps without a sponge 2779 x 8574 1.34 / 1.24 / 1.18 / 1.13 / 1.08 / 1.03 / 1.00.
+// Periodic grids cut nothing: 4/3 where the four-step FP32 BGK launch waits for HBM in part, 3/2
+// elsewhere.
 int outer_weight(const lb_ctx *c, int K) {
-    if (c->cfg.boundary != LB_PERIODIC) return c->cfg.sponge_width > 0 ? 13 : 12;
+    if (c->cfg.boundary != LB_PERIODIC) {
+        if (c->Q == 9) return 12;
+        if (c->cfg.sponge_width > 0) return 13;
+        return K == 6 ? 14 : c->cfg.storage == LB_BF16 ? 9 : 12;
+    }
     return c->Q == 5 && K <= 4 && c->cfg.storage == LB_F32 && c->cfg.collision == LB_BGK ? 8 : 9;
 }
 
@@ -196,9 +203,9 @@ static lb_status tile_launch(lb_ctx *ctx, const StepArgs &a, const WaveArgs &rec
     t.K = K;
     const int tiles = tiles_of(ctx, K, &t.tx), ctas = tiles <= sm_count() ? 1 : 2;
     const int ck = collision_kind(ctx);
-    const bool rho = a.rho_out != nullptr;
-    const TileFn fn = ctx->cfg.storage == LB_BF16 ? pick_tile_bf16(ck, rho, ctas)
-                                                  : pick_tile_f32(ck, rho, ctas);
+    const bool rho = a.rho_out != nullptr, per = ctx->cfg.boundary == LB_PERIODIC;
+    const TileFn fn = ctx->cfg.storage == LB_BF16 ? pick_tile_bf16(ck, rho, ctas, per)
+                                                  : pick_tile_f32(ck, rho, ctas, per);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(Shared));
     if (e == cudaSuccess)

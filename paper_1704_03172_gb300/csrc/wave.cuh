@@ -46,6 +46,7 @@ constexpr int kRing = 3;    // row slots per warp
 constexpr int kMedRow = 32 * 16;  // bytes of a row in the medium ring: per lane m, m, f, f
 
 enum { kLossless = 0, kBgk = 1, kMrt = 2 };  // D2Q5 BGK with omega = 2; BGK; MRT
+enum { kZeroGhost = 0, kPeriodic = 1, kEither = 2 };  // a kernel's boundary (kEither: WaveArgs::per)
 
 // recomputed columns on each side: K rounded up to whole lanes
 __host__ __device__ constexpr int halo(int K) { return (K + 1) / 2 * 2; }
@@ -604,8 +605,8 @@ __device__ __forceinline__ void iterate(const StepArgs &a, const WaveArgs &w, co
     at.eta2 += a.pitch;
     // Cuts at zero-ghost faces (cut_left), in one place ahead of the levels, which are short of
     // registers and instruction fetch (two-layer 4096^2, 200 steps: 8390 us with the cuts in each
-    // level, 10530 with levels of their own for the warps at a face, 7410 here and 6690 once those
-    // warps' rows count more, outer_weight; 6840 without cuts and at the rows' old weight)
+    // level, 10530 with levels of their own for the warps at a face, 7410 here, 6690 once those warps'
+    // rows count more, outer_weight, and the kernel knows its boundary; 6850 without cuts)
     if (!FAST && !T.per && (T.face || r <= K || r >= a.ny)) {  // warp-uniform
 #pragma unroll
         for (int l = 0; l < K; l++) {
@@ -683,7 +684,7 @@ __device__ __forceinline__ void iterate(const StepArgs &a, const WaveArgs &w, co
 
 // One strip and row chunk of a grid.  smem: this warp's warp_bytes(); tab: room for the CTA's
 // medium table.  Every warp of the CTA calls it (one barrier); those beyond the tasks do nothing.
-template <int Q, int CK, int K, bool REC, typename ST, bool ROUND>
+template <int Q, int CK, int K, bool REC, typename ST, bool ROUND, int BOUND>
 __device__ __forceinline__ void sweep(const StepArgs &a, const WaveArgs &w, int task,
                                       unsigned char *smem, float *tab) {
     if (a.mid)  // 8 B a thread
@@ -704,7 +705,7 @@ __device__ __forceinline__ void sweep(const StepArgs &a, const WaveArgs &w, int 
         bx = w.edge_l + (task - ne) - by * inner;
     }
     T.lane = threadIdx.x & 31;
-    T.per = w.per != 0;
+    T.per = BOUND == kEither ? w.per != 0 : BOUND == kPeriodic;
     T.gx = bx * out_cols(K) - halo(K) + 2 * T.lane;
     T.gxw = T.gx;
     T.live = true;
@@ -816,7 +817,7 @@ __device__ __forceinline__ void sweep(const StepArgs &a, const WaveArgs &w, int 
 // resident CTAs per SM the registers are cut for
 template <int Q, int K, typename ST> constexpr int min_ctas() { return Q == 9 ? (K > 2 ? (sizeof(ST) == 4 ? 2 : 3) : 3) : K > 4 ? 3 : 4; }
 
-template <int Q, int CK, int K, bool REC, typename ST, bool ROUND>
+template <int Q, int CK, int K, bool REC, typename ST, bool ROUND, int BOUND>
 __global__ void __launch_bounds__(kCtaThreads, min_ctas<Q, K, ST>())
     wave_kernel(const StepArgs a, const WaveArgs w) {
     // No early launch of dependents: the next grid's CTAs would take the slots of this grid's
@@ -828,7 +829,7 @@ __global__ void __launch_bounds__(kCtaThreads, min_ctas<Q, K, ST>())
     extern __shared__ __align__(16) unsigned char smem[];
     float *tab = reinterpret_cast<float *>(smem + kWarpsPerCta * warp_bytes<Q, K, ST>());
     const int wi = threadIdx.x >> 5;
-    sweep<Q, CK, K, REC, ST, ROUND>(a, w, blockIdx.x * kWarpsPerCta + wi, smem + wi * warp_bytes<Q, K, ST>(), tab);
+    sweep<Q, CK, K, REC, ST, ROUND, BOUND>(a, w, blockIdx.x * kWarpsPerCta + wi, smem + wi * warp_bytes<Q, K, ST>(), tab);
 }
 
 template <bool MRT, int K, typename ST, bool ROUND>
@@ -838,12 +839,12 @@ __device__ __forceinline__ void sweep_shot(const StepArgs &a, const WaveArgs &w,
     const int wi = threadIdx.x >> 5, task = block * kWarpsPerCta + wi;
     unsigned char *mine = smem + wi * warp_bytes<5, K, ST>();
     if constexpr (MRT) {
-        sweep<5, kMrt, K, true, ST, ROUND>(a, w, task, mine, tab);
+        sweep<5, kMrt, K, true, ST, ROUND, kEither>(a, w, task, mine, tab);
     } else {  // (block-uniform)
         if (a.omega == 2.f)
-            sweep<5, kLossless, K, true, ST, ROUND>(a, w, task, mine, tab);
+            sweep<5, kLossless, K, true, ST, ROUND, kEither>(a, w, task, mine, tab);
         else
-            sweep<5, kBgk, K, true, ST, ROUND>(a, w, task, mine, tab);
+            sweep<5, kBgk, K, true, ST, ROUND, kEither>(a, w, task, mine, tab);
     }
 }
 

@@ -2,7 +2,7 @@
 #include "wave_host.h"
 
 namespace lbwave {
-WavePick pick_d2q9_f32(int ck, int K, bool rec) {
-    return K == 4 ? pick_rec<9, 4, float, false>(ck, rec) : pick_rec<9, 2, float, false>(ck, rec);
+WavePick pick_d2q9_f32(int ck, int K, bool rec, bool per) {
+    return K == 4 ? pick_rec<9, 4, float, false>(ck, rec, per) : pick_rec<9, 2, float, false>(ck, rec, per);
 }
 }  // namespace lbwave

@@ -2,8 +2,8 @@
 #include "wave_host.h"
 
 namespace lbwave {
-WavePick pick_d2q9_bf16(int ck, int K, bool rec) {
-    return K == 4 ? pick_rec<9, 4, __nv_bfloat16, true>(ck, rec)
-                  : pick_rec<9, 2, __nv_bfloat16, true>(ck, rec);
+WavePick pick_d2q9_bf16(int ck, int K, bool rec, bool per) {
+    return K == 4 ? pick_rec<9, 4, __nv_bfloat16, true>(ck, rec, per)
+                  : pick_rec<9, 2, __nv_bfloat16, true>(ck, rec, per);
 }
 }  // namespace lbwave

@@ -2,5 +2,5 @@
 #include "wave_host.h"
 
 namespace lbwave {
-WavePick pick_d2q5_f16(int ck, bool rec) { return pick_rec<5, 2, __half, true>(ck, rec); }
+WavePick pick_d2q5_f16(int ck, bool rec, bool per) { return pick_rec<5, 2, __half, true>(ck, rec, per); }
 }  // namespace lbwave
