@@ -537,6 +537,8 @@ extern "C" lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *g
         if (ctx->nrec > 0 && ctx->ckpt_t0 != ctx->t_rec0)
             return fail(ctx, LB_ESTATE, "receivers must be set at the checkpointed start time");
     }
+    if (ctx->Q == 5 && ctx->nrec > 0 && !ctx->row_off)
+        return fail(ctx, LB_ESTATE, "the receivers' row lists could not be allocated");
     const int Q = ctx->Q;
     // forward states (checkpoints, replays) in the storage type; adjoint states FP32
     const size_t plane = (size_t)ctx->ny * ctx->pitch, sbytes = (size_t)Q * plane * ctx->ebytes,
@@ -605,26 +607,9 @@ extern "C" lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *g
                                              (int)tb_smem);
         if (e != cudaSuccess) return release(cuda_fail(ctx, e, "blocked adjoint shared memory"));
     }
-    // D2Q5: the wavefront sweep (adjoint5.cu), kAdj5Levels levels per launch, receivers by row
+    // D2Q5: tiles (tile_adj.cu) or the wavefront sweep (adjoint5.cu), several levels per launch,
+    // with the receivers by row of the context
     const bool wave = Q == 5;
-    const int *row_off = nullptr, *row_x = nullptr, *row_id = nullptr;
-    if (wave && ctx->nrec > 0) {
-        std::vector<int> off, xs, ids;
-        adj5_row_lists(ctx, off, xs, ids);
-        int *o = static_cast<int *>(grab(off.size() * sizeof(int)));
-        int *x = static_cast<int *>(grab(xs.size() * sizeof(int)));
-        int *i = static_cast<int *>(grab(ids.size() * sizeof(int)));
-        if (!o || !x || !i) return release(fail(ctx, LB_ENOMEM, "row receiver lists"));
-        cudaMemcpyAsync(o, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
-        cudaMemcpyAsync(x, xs.data(), xs.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
-        cudaMemcpyAsync(i, ids.data(), ids.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream);
-        // the host vectors go out of scope: the copies must have read them
-        cudaError_t e = cudaStreamSynchronize(ctx->stream);
-        if (e != cudaSuccess) return release(cuda_fail(ctx, e, "row receiver lists"));
-        row_off = o;
-        row_x = x;
-        row_id = i;
-    }
     std::vector<int> reg_off;
     std::vector<int2> reg_ent;
     if (!wave && ctx->nrec > 0) {
@@ -697,8 +682,7 @@ extern "C" lb_status lb_adjoint(lb_ctx *ctx, const float *dJdp, int nt, float *g
                 if (e != cudaSuccess && rst == LB_OK) rst = cuda_fail(ctx, e, "tiled adjoint");
                 m -= Kt;
             } else if (wave && m + 1 >= kAdj5Levels) {  // levels sa + m .. sa + m - K + 1, wavefront
-                const cudaError_t e =
-                    adj5_launch(ctx, a, d, d.rho, a.t, row_off, row_x, row_id);
+                const cudaError_t e = adj5_launch(ctx, a, d, d.rho, a.t);
                 if (e != cudaSuccess && rst == LB_OK) rst = cuda_fail(ctx, e, "wavefront adjoint");
                 m -= kAdj5Levels;
             } else if (!wave && m + 1 >= Ka) {  // levels sa + m .. sa + m - Ka + 1 in one launch

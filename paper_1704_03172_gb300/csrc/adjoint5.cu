@@ -22,7 +22,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <vector>
 
 #include "adjoint_site.cuh"
 #include "lb_kernels.cuh"
@@ -318,33 +317,10 @@ __global__ void __launch_bounds__(kWS, 3) adj5_kernel(const StepArgs a, const Ad
 using namespace lbadj5;
 using namespace lbrt;
 
-// Receivers by row for the wavefront sweep: offsets [ny + 1], x ascending within a row.
-void adj5_row_lists(const lb_ctx *ctx, std::vector<int> &off, std::vector<int> &xs,
-                    std::vector<int> &ids) {
-    const int n = ctx->nrec;
-    off.assign((size_t)ctx->ny + 1, 0);
-    std::vector<int> order(n);
-    for (int r = 0; r < n; r++) {
-        off[(size_t)ctx->rec_xy[2 * r + 1] + 1]++;
-        order[r] = r;
-    }
-    for (size_t k = 1; k < off.size(); k++) off[k] += off[k - 1];
-    const int *xy = ctx->rec_xy.data();
-    std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
-        return xy[2 * p + 1] != xy[2 * q + 1] ? xy[2 * p + 1] < xy[2 * q + 1] : xy[2 * p] < xy[2 * q];
-    });
-    xs.assign(std::max(n, 1), 0);
-    ids.assign(std::max(n, 1), 0);
-    for (int k = 0; k < n; k++) {
-        xs[k] = xy[2 * order[k]];
-        ids[k] = order[k];
-    }
-}
-
 // K = kAdj5Levels adjoint levels t_hi .. t_hi - K + 1 from d.lam_in into d.lam_out, with
 // rho^t_hi at rho_hi (rho^t at rho_hi - (t_hi - t) plane), on ctx's stream.
 cudaError_t adj5_launch(lb_ctx *ctx, const StepArgs &a, const AdjArgs &d, const float *rho_hi,
-                        long long t_hi, const int *row_off, const int *rec_x, const int *rec_id) {
+                        long long t_hi) {
     constexpr int K = kAdj5Levels;
     const bool mrt = ctx->cfg.collision == LB_MRT;
     auto fn = mrt ? adj5_kernel<true, K> : adj5_kernel<false, K>;
@@ -364,9 +340,9 @@ cudaError_t adj5_launch(lb_ctx *ctx, const StepArgs &a, const AdjArgs &d, const 
     Adj5Args b;
     b.rho_hi = rho_hi;
     b.t_hi = t_hi;
-    b.row_off = row_off;
-    b.rec_x = rec_x;
-    b.rec_id = rec_id;
+    b.row_off = ctx->nrec > 0 ? ctx->row_off : nullptr;
+    b.rec_x = ctx->row_x;
+    b.rec_id = ctx->row_id;
     b.H = std::max(1, (ctx->ny + chunks - 1) / chunks);
     b.per = ctx->cfg.boundary == LB_PERIODIC ? 1 : 0;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

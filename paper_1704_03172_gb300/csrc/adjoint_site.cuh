@@ -141,15 +141,11 @@ struct AdjArgs {
 
 }  // namespace lbadj
 
-// The D2Q5 wavefront reverse sweep (adjoint5.cu): levels per launch, the receivers' row lists
-// ([ny + 1] offsets, x ascending, receiver ids) and the launch of kAdj5Levels levels
-// t_hi .. t_hi - kAdj5Levels + 1 (rho^t at rho_hi - (t_hi - t) plane) on ctx's stream.
+// The D2Q5 wavefront reverse sweep (adjoint5.cu): levels per launch, and the launch of kAdj5Levels
+// levels t_hi .. t_hi - kAdj5Levels + 1 (rho^t at rho_hi - (t_hi - t) plane) on ctx's stream.
 constexpr int kAdj5Levels = 4;
-void adj5_row_lists(const lb_ctx *ctx, std::vector<int> &off, std::vector<int> &xs,
-                    std::vector<int> &ids);
 cudaError_t adj5_launch(lb_ctx *ctx, const lbk::StepArgs &a, const lbadj::AdjArgs &d,
-                        const float *rho_hi, long long t_hi, const int *row_off, const int *rec_x,
-                        const int *rec_id);
+                        const float *rho_hi, long long t_hi);
 
 // The same on register tiles (tile_adj.cu): levels of the next launch of n wanted ones (0: the
 // grid is the wavefront's), and the launch of K levels
