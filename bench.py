@@ -44,19 +44,12 @@ ELEM_BYTES = {"f32": 4, "bf16": 2, "f16": 2}
 KERNEL_SOURCES = {
     "lbk::step_kernel": ("lb_kernels.cuh",),
     "stream_step_kernel": ("lb_kernels.cuh", "aa_sites.cuh", "stream_step.cu"),
-    "lbtb5::tb5_kernel": ("lb_kernels.cuh", "tblock5.cuh"),
 }
 NCU_TRAFFIC = {
     ("lbk::step_kernel<5,false,false,float>", True):
         (638.5e6, "df1c40b8bd02", "profiles/step_kernel_d2q5_f32_4096.md"),
     ("stream_step_kernel<5,false,false,__nv_bfloat16>", True):
         (300.3e6, "3a52a69fc363", "profiles/stream_step_kernel_d2q5_bf16_4096.md"),
-    ("lbtb5::tb5_kernel<false,4,false,float>", True):
-        (656.4e6, "be28d81b9dd6", "profiles/tb5_kernel_d2q5_4096.md"),
-    ("lbtb5::tb5_kernel<false,4,false,__nv_bfloat16>", True):
-        (314.8e6, "be28d81b9dd6", "profiles/tb5_kernel_d2q5_4096.md"),
-    ("lbtb5::tb5_kernel<false,8,false,float>", True):
-        (671.9e6, "be28d81b9dd6", "profiles/tb5_kernel_d2q5_4096.md"),
 }
 
 
@@ -203,8 +196,33 @@ def _make_sim(LBSim, wl, nt_cap):
     return sim
 
 
+def steps_per_launch(steps, launches, storage, streaming="ab"):
+    """Steps that one launch takes on average, from the kernels lb_step launched (lb_info; 0 where it
+    does not count them: one step each).  FP16 launches are followed by the scales' update, launches of
+    two FP16 steps by that and by one more that mends them: with s launches of one step and f of two,
+    2 s + 3 f launches take s + 2 f steps."""
+    if launches <= 0 or streaming == "aa":
+        return 1.0
+    if storage == "f16":
+        launches -= steps
+    return steps / launches
+
+
+def hbm_use(Q, storage, indexed, sites, steps, fused, sec):
+    """Memory rates of `steps` steps in launches of `fused` steps, each of which has to read and write
+    the state and read the medium once: GB/s, that over the measured copy, and what one launch per
+    step would have had to move in the same time (GB/s; it may exceed what memory can do)."""
+    once = bytes_per_site(Q, storage, indexed) * sites / 1e9
+    gbs = once * steps / fused / sec
+    return {"achieved_gbs": round(gbs, 1), "frac_of_measured_hbm": round(gbs / _peaks()[0], 4),
+            "steps_per_launch": round(fused, 2),
+            "one_step_equivalent_gbs": round(once * steps / sec, 1)}
+
+
 def _time_steps(torch, sim, steps, warmup):
+    """Seconds of `steps` steps after `warmup`, and the kernels they launched."""
     sim.step(warmup)
+    launches = sim.info()[6]
     torch.cuda.synchronize()
     stream = sim.stream
     e0 = torch.cuda.Event(enable_timing=True)
@@ -213,7 +231,7 @@ def _time_steps(torch, sim, steps, warmup):
     sim.step(steps)
     e1.record(stream)
     torch.cuda.synchronize()
-    return e0.elapsed_time(e1) / 1e3
+    return e0.elapsed_time(e1) / 1e3, int(sim.info()[6] - launches)
 
 
 def _variant(torch, LBSim, lattice, storage, collision, steps, warmup, time_block=1,
@@ -223,18 +241,17 @@ def _variant(torch, LBSim, lattice, storage, collision, steps, warmup, time_bloc
     wl["streaming"] = streaming
     sim = _make_sim(LBSim, wl, steps + warmup)
     try:
-        # the D2Q9 tile-blocked kernel reads eta^2 per site; the others the medium index
-        indexed = _indexed(sim) and (time_block <= 1 or lattice == 5)
-        sec = _time_steps(torch, sim, steps, warmup)
+        indexed = _indexed(sim)
+        sec, launches = _time_steps(torch, sim, steps, warmup)
     finally:
         sim.close()
     sites = N_GRID * N_GRID
     glups = sites * steps / sec / 1e9
-    bps = bytes_per_site(lattice, storage, indexed)
-    out = {"glups": round(glups, 2), "bytes_per_site": bps,
-           "achieved_gbs": round(glups * bps, 1), "ms_per_step": round(sec / steps * 1e3, 4)}
+    out = {"glups": round(glups, 2), "bytes_per_site": bytes_per_site(lattice, storage, indexed),
+           "ms_per_step": round(sec / steps * 1e3, 4),
+           **hbm_use(lattice, storage, indexed, sites, steps,
+                     steps_per_launch(steps, launches, storage, streaming), sec)}
     if streaming == "aa":
-        out["frac_of_measured_hbm"] = round(glups * bps / _peaks()[0], 4)
         out["population_gb"] = round(lattice * sites * ELEM_BYTES[storage] / 1e9, 3)
         out["streaming"] = "in place: one population buffer (two-buffer form: twice this)"
     return out
@@ -262,13 +279,12 @@ def _layered_variant(torch, LBSim, storage, steps, warmup, n=8192):
         sim.set_receivers(wl["receivers"], steps + warmup)
         sim.init_pressure(None)
         indexed = _indexed(sim)
-        sec = _time_steps(torch, sim, steps, warmup)
+        sec, launches = _time_steps(torch, sim, steps, warmup)
     finally:
         sim.close()
     glups = n * n * steps / sec / 1e9
-    bps = bytes_per_site(5, storage, indexed)
-    return {"glups": round(glups, 2), "bytes_per_site": bps, "achieved_gbs": round(glups * bps, 1),
-            "frac_of_measured_hbm": round(glups * bps / _peaks()[0], 4),
+    return {"glups": round(glups, 2), "bytes_per_site": bytes_per_site(5, storage, indexed),
+            **hbm_use(5, storage, indexed, n * n, steps, steps_per_launch(steps, launches, storage), sec),
             "ms_per_step": round(sec / steps * 1e3, 4), "grid": f"{n}^2", "steps": steps,
             "state_gb": round(2 * 5 * n * n * ELEM_BYTES[storage] / 1e9, 2)}
 
@@ -284,7 +300,7 @@ def _refined_variant(torch, LBSim, steps, warmup):
     sim.set_receivers(wl["receivers"], steps + warmup)
     sim.init_pressure(None)
     try:
-        sec = _time_steps(torch, sim, steps, warmup)
+        sec, _ = _time_steps(torch, sim, steps, warmup)
     finally:
         sim.close()
     nf = 2 * wl["patch"][2] + 1
@@ -383,7 +399,7 @@ def _l2_variant(torch, LBSim, n, storage, steps, warmup=50, time_block=1):
     wl["time_block"] = time_block
     sim = _make_sim(LBSim, wl, steps + warmup)
     try:
-        sec = _time_steps(torch, sim, steps, warmup)
+        sec, _ = _time_steps(torch, sim, steps, warmup)
         pitch = sim.info()[1]
     finally:
         sim.close()
@@ -405,7 +421,7 @@ def _nested_variant(torch, LBSim, steps, warmup):
     sim.set_receivers(wl["receivers"], steps + warmup)
     sim.init_pressure(None)
     try:
-        sec = _time_steps(torch, sim, steps, warmup)
+        sec, _ = _time_steps(torch, sim, steps, warmup)
     finally:
         sim.close()
     n1 = 2 * wl["patches"][0][2] + 1
@@ -522,12 +538,12 @@ def _d3q7_variant(torch, LBSim, storage, n=256, steps=300, warmup=10):
         sim.set_receivers(rec, steps + warmup)
         sim.init_pressure(None)
         indexed = _indexed(sim)
-        sec = _time_steps(torch, sim, steps, warmup)
+        sec, launches = _time_steps(torch, sim, steps, warmup)
     finally:
         sim.close()
     glups = n ** 3 * steps / sec / 1e9
-    bps = 2 * 7 * ELEM_BYTES[storage] + (1 if indexed else 4)
-    return {"glups": round(glups, 2), "bytes_per_site": bps, "achieved_gbs": round(glups * bps, 1),
+    return {"glups": round(glups, 2), "bytes_per_site": bytes_per_site(7, storage, indexed),
+            **hbm_use(7, storage, indexed, n ** 3, steps, steps_per_launch(steps, launches, storage), sec),
             "ms_per_step": round(sec / steps * 1e3, 4), "grid": f"{n}^3"}
 
 
@@ -971,9 +987,8 @@ def run_ours(args):
         return 0
     peak, peak_kind = _peaks()
     # lb_step takes several steps per launch where its fused kernels are faster
-    fused = args.steps / max(launches, 1)
-    bps = bytes_per_site(args.lattice, args.storage, indexed)
-    achieved = bps * sites * args.steps / sec / 1e9   # algorithmic one-step bytes per update
+    fused = steps_per_launch(args.steps, launches, args.storage)
+    use = hbm_use(args.lattice, args.storage, indexed, sites, args.steps, fused, sec)
     staged = (args.step_kernel == "staged" or
               (args.step_kernel == "auto" and args.storage != "f32"))
     st_name = dict(f32='float', bf16='__nv_bfloat16', f16='__half')[args.storage]
@@ -998,12 +1013,15 @@ def run_ours(args):
                    "l2": "inputs larger than L2 (each population buffer >= 168 MB; 129 MB L2)",
                    "medium": "1-byte medium index + eta^2 table" if indexed
                              else "eta^2 per site (FP32)"},
-        "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak,
-                     "peak_kind": peak_kind, "unit": "GB/s", "frac": round(achieved / peak, 4),
+        "roofline": {"bound": "hbm" if fused <= 1 else "issue", "achieved": use["achieved_gbs"],
+                     "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
+                     "frac": use["frac_of_measured_hbm"],
                      "traffic": traffic, "traffic_source": traffic_src, "kernel": kname,
-                     "algorithmic_bytes_per_launch": round(bps * sites * fused),
-                     "note": "achieved counts the one-step algorithmic bytes of every fused "
-                             "step (one-step equivalent bandwidth)"
+                     "algorithmic_bytes_per_launch":
+                         round(bytes_per_site(args.lattice, args.storage, indexed) * sites),
+                     "one_step_equivalent_gbs": use["one_step_equivalent_gbs"],
+                     "note": "achieved counts one read and one write of the state per launch of "
+                             f"{fused:.1f} steps; one_step_equivalent_gbs counts them per step"
                      if fused > 1 else "one launch per step"},
         "gpu_launches": launches,
         "clocks": clk.summary(),
