@@ -197,7 +197,7 @@ int wave_batch_rows(lb_ctx *const *ctxs, int n);
 bool wave_batch_round(lb_ctx *const *ctxs, int n);
 int wave_batch_blocks(const lb_ctx *ctx, int H);
 int wave_batch_fill(lb_ctx *const *ctxs, int n, int H, void *h);
-cudaError_t wave_batch_launch(const void *d, int n, int blocks, bool mrt, bool round,
+cudaError_t wave_batch_launch(const void *d, int n, int blocks, bool mrt, bool round, bool per,
                               cudaStream_t stream);
 // D2Q5 BF16 blocks of cfg.time_block steps with FP32 between them (tblock5.cu)
 lb_status tb5_launch_args(lb_ctx *ctx, const lbk::StepArgs &a, int K);

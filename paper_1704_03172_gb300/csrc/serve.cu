@@ -392,17 +392,18 @@ void pass(lb_server *S) {
         }
     }
     batched.swap(rest);
-    // one launch for FP32 and BF16 shots; a rho tape wants the BF16 of every step
+    // one launch for FP32 and BF16 shots of a boundary; a rho tape wants the BF16 of every step
     auto tb_key = [&](const Req *r) {
-        return std::pair<bool, bool>(r->cfg.collision == LB_MRT,
-                                     round || (r->cfg.storage == LB_BF16 && r->ctx->rho_tape));
+        return std::tuple<bool, bool, bool>(r->cfg.collision == LB_MRT,
+                                            round || (r->cfg.storage == LB_BF16 && r->ctx->rho_tape),
+                                            r->cfg.boundary == LB_PERIODIC);
     };
     std::stable_sort(tbs.begin(), tbs.end(),
                      [&](const Req *a, const Req *b) { return tb_key(a) < tb_key(b); });
     struct TbLaunch {
         size_t off;
         int n, blocks;
-        bool mrt, round;
+        bool mrt, round, per;
         size_t g0, g1;
     };
     std::vector<TbLaunch> tb_launches;
@@ -430,8 +431,8 @@ void pass(lb_server *S) {
                 const int n = (int)(g1 - g0);
                 const int blocks =
                     wave_batch_fill(cs.data(), n, tb_rows, static_cast<char *>(S->h_tb) + off);
-                const auto [mrt, rounds] = tb_key(tbs[g0]);
-                tb_launches.push_back({off, n, blocks, mrt, rounds, g0, g1});
+                const auto [mrt, rounds, per] = tb_key(tbs[g0]);
+                tb_launches.push_back({off, n, blocks, mrt, rounds, per, g0, g1});
                 off += wave_batch_bytes(n);
                 g0 = g1;
             }
@@ -514,7 +515,7 @@ void pass(lb_server *S) {
     }
     for (const TbLaunch &L : tb_launches) {  // time-blocked blocks of K steps
         e = wave_batch_launch(static_cast<char *>(S->d_tb) + L.off, L.n, L.blocks, L.mrt, L.round,
-                              S->stream);
+                              L.per, S->stream);
         if (e != cudaSuccess) {
             const std::string msg = std::string("time-blocked batch: ") + cudaGetErrorString(e);
             set_err(S, msg);

@@ -26,7 +26,7 @@ WavePick pick_d2q5_f32(int ck, int K, bool rec, bool per) {
                                      : pick_one<5, kBgk, 6, false, float, false>(per);
     return K == 4 ? pick_rec<5, 4, float, false>(ck, rec, per) : pick_rec<5, 2, float, false>(ck, rec, per);
 }
-WaveBatchFn pick_batch_fp32(bool mrt) { return pick_batch<false>(mrt); }
+WaveBatchFn pick_batch_fp32(bool mrt, bool per) { return pick_batch<false>(mrt, per); }
 }  // namespace lbwave
 
 namespace lbrt {
@@ -340,7 +340,9 @@ BatchLayout batch_layout(void *base, int n) {
 }
 // tasks and shape of one shot at about H rows per chunk
 int batch_shape(const lb_ctx *c, int H, WaveArgs &w) {
-    w.outer = outer_weight(c, kServeSteps);
+    // (9 sixths on small shots, whose chunks are short already: 32 of 256^2 568 shots/s against 461 at
+    // 10, of 2048^2 37.8 against 38.7 at 11)
+    w.outer = c->ny < 1024 ? 9 : 11;
     strips_of(w, c->nx, kServeSteps, c->cfg.sponge_width, c->cfg.boundary == LB_PERIODIC);
     H = std::max(1, std::min(c->ny, H));
     return (int)set_chunks(w, c->ny, (c->ny + H - 1) / H);
@@ -378,7 +380,7 @@ int wave_batch_rows(lb_ctx *const *ctxs, int n) {
     }
     const long long slots1 = (long long)sm_count() * kWarpsPerCta;
     long long cost = -1, best = 1;
-    for (int m = 1; m <= 4; m++) {
+    for (int m = 1; m <= 2; m++) {  // (three: 512^2 291 shots/s against 357, 2048^2 35.5 against 37.8)
         const long long H = std::min<long long>(ny, (rows + m * slots1 - 1) / (m * slots1));
         const long long c = (H + 2 * kServeSteps) * (4 + m);
         if (cost < 0 || c < cost) cost = c, best = H;
@@ -446,9 +448,9 @@ int wave_batch_fill(lb_ctx *const *ctxs, int n, int H, void *h) {
 }
 
 cudaError_t wave_batch_launch(const void *d, int n, int blocks, bool mrt, bool round,
-                              cudaStream_t stream) {
+                              bool per, cudaStream_t stream) {
     if (n < 1 || blocks < 1) return cudaErrorInvalidValue;
-    const WaveBatchFn fn = round ? pick_batch_round(mrt) : pick_batch_fp32(mrt);
+    const WaveBatchFn fn = round ? pick_batch_round(mrt, per) : pick_batch_fp32(mrt, per);
     constexpr int smem = cta_bytes<5, kServeSteps, float>();
     static_assert(smem >= cta_bytes<5, kServeSteps, __nv_bfloat16>(), "room for either storage");
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

@@ -832,19 +832,19 @@ __global__ void __launch_bounds__(kCtaThreads, min_ctas<Q, K, ST>())
     sweep<Q, CK, K, REC, ST, ROUND, BOUND>(a, w, blockIdx.x * kWarpsPerCta + wi, smem + wi * warp_bytes<Q, K, ST>(), tab);
 }
 
-template <bool MRT, int K, typename ST, bool ROUND>
+template <bool MRT, int K, typename ST, bool ROUND, int BOUND>
 __device__ __forceinline__ void sweep_shot(const StepArgs &a, const WaveArgs &w, int block,
                                            unsigned char *smem) {
     float *tab = reinterpret_cast<float *>(smem + kWarpsPerCta * warp_bytes<5, K, ST>());
     const int wi = threadIdx.x >> 5, task = block * kWarpsPerCta + wi;
     unsigned char *mine = smem + wi * warp_bytes<5, K, ST>();
     if constexpr (MRT) {
-        sweep<5, kMrt, K, true, ST, ROUND, kEither>(a, w, task, mine, tab);
+        sweep<5, kMrt, K, true, ST, ROUND, BOUND>(a, w, task, mine, tab);
     } else {  // (block-uniform)
         if (a.omega == 2.f)
-            sweep<5, kLossless, K, true, ST, ROUND, kEither>(a, w, task, mine, tab);
+            sweep<5, kLossless, K, true, ST, ROUND, BOUND>(a, w, task, mine, tab);
         else
-            sweep<5, kBgk, K, true, ST, ROUND, kEither>(a, w, task, mine, tab);
+            sweep<5, kBgk, K, true, ST, ROUND, BOUND>(a, w, task, mine, tab);
     }
 }
 
@@ -852,9 +852,12 @@ __device__ __forceinline__ void sweep_shot(const StepArgs &a, const WaveArgs &w,
 // [first[k], first[k + 1]) and reads its own descriptors (the served batches).  FP32 and BF16 shots
 // share the launch (ROUND: the BF16 ones round at every step): a few small shots leave most of
 // the chip idle, and a launch of K steps takes its 10 us
-// however few they are (24 shots of 256^2 to 1024^2, 400 steps: 41 ms against 47 apart).
-template <bool MRT, int K, bool ROUND>
-__global__ void __launch_bounds__(kCtaThreads, min_ctas<5, K, float>())
+// however few they are (24 shots of 256^2 to 1024^2, 400 steps: 41 ms against 47 apart).  Shots of one
+// boundary and three CTAs per SM (146 registers): one kernel for both boundaries spills 572 B at four,
+// one for each 356 B (32 shots of 512^2: 274 and 266 shots/s against 357).
+constexpr int kBatchCtas = 3;
+template <bool MRT, int K, bool ROUND, int BOUND>
+__global__ void __launch_bounds__(kCtaThreads, kBatchCtas)
     wave_batch_kernel(const StepArgs *__restrict__ args, const WaveArgs *__restrict__ waves,
                       const int *__restrict__ first, int nshots) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -877,9 +880,9 @@ __global__ void __launch_bounds__(kCtaThreads, min_ctas<5, K, float>())
     }
     __syncthreads();
     if (sw.bf16)  // (block-uniform)
-        sweep_shot<MRT, K, __nv_bfloat16, ROUND>(sa, sw, s_blk, smem);
+        sweep_shot<MRT, K, __nv_bfloat16, ROUND, BOUND>(sa, sw, s_blk, smem);
     else
-        sweep_shot<MRT, K, float, false>(sa, sw, s_blk, smem);
+        sweep_shot<MRT, K, float, false, BOUND>(sa, sw, s_blk, smem);
 }
 
 using WaveFn = void (*)(const StepArgs, const WaveArgs);

@@ -38,11 +38,14 @@ WavePick pick_d2q5_f16(int ck, bool rec, bool per);          // wave_f16.cu: two
 WavePick pick_d2q9_f32(int ck, int K, bool rec, bool per);   // wave9.cu
 WavePick pick_d2q9_bf16(int ck, int K, bool rec, bool per);  // wave9_bf16.cu
 
-template <bool ROUND> WaveBatchFn pick_batch(bool mrt) {
-    return mrt ? wave_batch_kernel<true, kServeSteps, ROUND>
-               : wave_batch_kernel<false, kServeSteps, ROUND>;
+template <bool ROUND> WaveBatchFn pick_batch(bool mrt, bool per) {
+    if (per)
+        return mrt ? wave_batch_kernel<true, kServeSteps, ROUND, kPeriodic>
+                   : wave_batch_kernel<false, kServeSteps, ROUND, kPeriodic>;
+    return mrt ? wave_batch_kernel<true, kServeSteps, ROUND, kZeroGhost>
+               : wave_batch_kernel<false, kServeSteps, ROUND, kZeroGhost>;
 }
-WaveBatchFn pick_batch_fp32(bool mrt);   // wave.cu: BF16 shots keep FP32 between a launch's steps
-WaveBatchFn pick_batch_round(bool mrt);  // wave_bf16.cu: they round at every step
+WaveBatchFn pick_batch_fp32(bool mrt, bool per);   // wave.cu: BF16 keeps FP32 between a launch's steps
+WaveBatchFn pick_batch_round(bool mrt, bool per);  // wave_bf16.cu: it is rounded at every step
 
 }  // namespace lbwave
