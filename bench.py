@@ -1013,7 +1013,7 @@ def run_ours(args):
                    "l2": "inputs larger than L2 (each population buffer >= 168 MB; 129 MB L2)",
                    "medium": "1-byte medium index + eta^2 table" if indexed
                              else "eta^2 per site (FP32)"},
-        "roofline": {"bound": "hbm" if fused <= 1 else "issue", "achieved": use["achieved_gbs"],
+        "roofline": {"bound": "hbm" if fused <= 1 else "latency", "achieved": use["achieved_gbs"],
                      "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
                      "frac": use["frac_of_measured_hbm"],
                      "traffic": traffic, "traffic_source": traffic_src, "kernel": kname,

@@ -172,7 +172,7 @@ lb_status stream_launch_aa(lb_ctx *ctx, const lbk::StepArgs &a, bool exchange, c
 lb_status tb_launch(lb_ctx *ctx, Fuse f);
 // in-place streaming (aa.cu): n steps of an LB_STREAM_AA context
 lb_status aa_step(lb_ctx *ctx, int n);
-// warp wavefront (wave.cu): 2, 4 or 6 steps of a D2Q5, 2 or 4 of a D2Q9 grid per launch, FP32 or
+// warp wavefront (wave.cu): 2, 4 or 6 steps of a D2Q5 (FP16: 2), 2 or 4 of a D2Q9 grid per launch, FP32 or
 // BF16 storage, with the one-step kernels' results bit for bit.  Whether a context has it, whether
 // it pays without being asked for, the steps the next launch takes of n wanted, the receivers' row
 // lists, and the launch

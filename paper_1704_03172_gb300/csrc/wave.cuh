@@ -12,15 +12,15 @@
 // x shifts take one shuffle per population.  Nothing is shared between warps: no barrier.
 //
 // What bounds it and why this shape: the one-step kernel is bound by HBM (41 B per D2Q5 site
-// and step), and K fused steps move 41 / K; what is left is instruction issue and the latency of
-// few warps.  A CTA-wide wavefront (256 columns, one a thread, x neighbours through shared memory
+// and step), and K fused steps move 41 / K; what is left is the latency of two to three warps per
+// scheduler, which fill 50 % (BF16: 67 %) of the issue slots.  A CTA-wide wavefront (256 columns, one a thread, x neighbours through shared memory
 // and a barrier per row) took 74 instructions per site and step and reached 316 GLUPS.  Here two
 // columns per lane go through packed FP32 operations (f32x2), neighbours come by shuffle, and
 // an iteration of four levels is about 225 instructions for 56 x 4 site updates.  Four columns
 // per lane needed 168 registers and twice the code: it spilled and starved on instruction
 // fetch (190 GLUPS where two columns gave 340).  GB300, 4096^2 / 8192^2, us a step before and
-// after: D2Q5 FP32 100.5 -> 29.0 / 398 -> 103 (K = 6), BF16 60.6 -> 30.8 / 256 -> 104 (K = 4),
-// MRT FP32 100.6 -> 32.4, D2Q9 FP32 184 -> 63.7 (K = 4).
+// after: D2Q5 FP32 100.5 -> 30.1 / 398 -> 100 (K = 6), BF16 60.6 -> 29.6 / 256 -> 103 (K = 4),
+// MRT FP32 100.6 -> 32.0, D2Q9 FP32 184 -> 63.6 (K = 4).
 //
 // Rows arrive by cp.async in a ring of kRing row slots per warp, kRing - 1 rows ahead, and
 // each lane reads only what it copied itself.  A second ring keeps the medium and the sponge
