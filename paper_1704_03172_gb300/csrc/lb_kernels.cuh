@@ -563,19 +563,15 @@ __device__ __forceinline__ void collide5(R g[5], R e2, const StepArgs &a) {
 // formed as in collide5.  One fused multiply-add per population instead of three
 // operations; the same values up to rounding.
 template <typename R>
-__device__ __forceinline__ void collide5_lossless_w(R g[5], R w1) {  // w1 = eta^2 / 4
+__device__ __forceinline__ void collide5_lossless(R g[5], R e2) {
     const R rho = g[0] + g[1] + g[2] + g[3] + g[4];
     const R jx = g[1] - g[3], jy = g[2] - g[4];
-    const R b = w1 * rho, eq0 = rho - R(4) * b;
+    const R b = R(0.25) * e2 * rho, eq0 = rho - R(4) * b;
     g[0] = fma(R(2), eq0, -g[0]);
     g[1] = fma(R(2), fma(R(0.5), jx, b), -g[1]);
     g[2] = fma(R(2), fma(R(0.5), jy, b), -g[2]);
     g[3] = fma(R(2), fma(R(-0.5), jx, b), -g[3]);
     g[4] = fma(R(2), fma(R(-0.5), jy, b), -g[4]);
-}
-template <typename R>
-__device__ __forceinline__ void collide5_lossless(R g[5], R e2) {
-    collide5_lossless_w(g, R(0.25) * e2);
 }
 
 // D2Q9 with the eta^2-scaled weights: w_{1..4} = eta^2 w1r, w_{5..8} = eta^2 w5r,

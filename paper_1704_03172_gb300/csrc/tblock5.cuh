@@ -116,7 +116,7 @@ __device__ __forceinline__ float tb5_e2(const StepArgs &a, const Tb5Thread &T, b
 // checks at all.
 // edgy (FAST, CTA-uniform): a column of the strip or a row of the iteration lies outside
 // the domain or in the sponge, so the fast path applies a per-site factor.
-template <bool MRT, int K, bool REC, typename ST, int P, bool FAST>
+template <bool MRT, int K, typename ST, int P, bool FAST>
 __device__ __forceinline__ void tb5_iter(const StepArgs &a, const Tb5Args &tb, const Tb5Thread &T,
                                          float (&W0)[2][K], float (&EE)[2][K], float (&G2)[2][K],
                                          float (&pre)[2][5], float (&pre_e2)[2], int r, int rend,
@@ -153,9 +153,6 @@ __device__ __forceinline__ void tb5_iter(const StepArgs &a, const Tb5Args &tb, c
         EE[P][l] = nE;
         const int y = r - l - 1;  // the row level l + 1 computes
         if (FAST) {
-            if (REC && T.own_col)
-                a.rho_out[l * a.rho_stride + (long long)y * a.pitch + T.gx] =
-                    g[0] + g[1] + g[2] + g[3] + g[4];
             if (!MRT && T.lossless)
                 collide5_lossless(g, e2);
             else
@@ -177,10 +174,9 @@ __device__ __forceinline__ void tb5_iter(const StepArgs &a, const Tb5Args &tb, c
             const bool mine = T.own_col && y >= T.Y0 && y < T.Y1;
             const bool row_rec = T.has_rec && y >= T.Y0 && y < T.Y1 &&
                                  tb.row_off[y + 1] > tb.row_off[y];  // warp-uniform
-            if ((REC && mine) || row_rec) {
+            if (row_rec) {
                 const float rho = g[0] + g[1] + g[2] + g[3] + g[4];
-                if (REC && mine) a.rho_out[l * a.rho_stride + (long long)y * a.pitch + T.gx] = rho;
-                if (row_rec && mine) {  // receivers of this site: binary search in the row
+                if (mine) {  // receivers of this site: binary search in the row
                     int lo = tb.row_off[y], hi = tb.row_off[y + 1];
                     while (lo < hi) {
                         const int mid = (lo + hi) >> 1;
@@ -220,9 +216,8 @@ __device__ __forceinline__ void tb5_iter(const StepArgs &a, const Tb5Args &tb, c
 }
 
 // The strip bx and row chunk by of one grid, K levels (the body of both kernels below).
-// REC: also record rho of every level of the own output sites (adjoint replays, rho tape).
 // xs_mem: [2][K][2][kWS + 2] floats of shared memory; s_tab: [kWS] floats.
-template <bool MRT, int K, bool REC, typename ST>
+template <bool MRT, int K, typename ST>
 __device__ __forceinline__ void tb5_body(const StepArgs &a, const Tb5Args &tb, int bx, int by,
                                          float *xs_mem, float *s_tab) {
     constexpr int OUT = kWS - 2 * K;
@@ -306,14 +301,14 @@ __device__ __forceinline__ void tb5_body(const StepArgs &a, const Tb5Args &tb, i
 #pragma unroll 1
     for (; r < rend; r += 2) {
         if (fast_ok(r))
-            tb5_iter<MRT, K, REC, ST, 0, true>(a, tb, T, W0, EE, G2, pre, pre_e2, r, rend, edgy(r));
+            tb5_iter<MRT, K, ST, 0, true>(a, tb, T, W0, EE, G2, pre, pre_e2, r, rend, edgy(r));
         else
-            tb5_iter<MRT, K, REC, ST, 0, false>(a, tb, T, W0, EE, G2, pre, pre_e2, r, rend, edgy(r));
+            tb5_iter<MRT, K, ST, 0, false>(a, tb, T, W0, EE, G2, pre, pre_e2, r, rend, edgy(r));
         if (r + 1 >= rend) break;
         if (fast_ok(r + 1))
-            tb5_iter<MRT, K, REC, ST, 1, true>(a, tb, T, W0, EE, G2, pre, pre_e2, r + 1, rend, edgy(r + 1));
+            tb5_iter<MRT, K, ST, 1, true>(a, tb, T, W0, EE, G2, pre, pre_e2, r + 1, rend, edgy(r + 1));
         else
-            tb5_iter<MRT, K, REC, ST, 1, false>(a, tb, T, W0, EE, G2, pre, pre_e2, r + 1, rend, edgy(r + 1));
+            tb5_iter<MRT, K, ST, 1, false>(a, tb, T, W0, EE, G2, pre, pre_e2, r + 1, rend, edgy(r + 1));
     }
 }
 
@@ -321,19 +316,19 @@ __device__ __forceinline__ void tb5_body(const StepArgs &a, const Tb5Args &tb, i
 // (<= 80 registers), two for the deep ones.
 template <int K> constexpr int tb5_min_blocks() { return K <= 4 ? 3 : 2; }
 
-template <bool MRT, int K, bool REC, typename ST>
+template <bool MRT, int K, typename ST>
 __global__ void __launch_bounds__(kWS, tb5_min_blocks<K>()) tb5_kernel(const StepArgs a,
                                                                       const Tb5Args tb) {
     pdl_trigger_and_wait();
     extern __shared__ float xs_mem[];
     __shared__ float s_tab[kWS];
-    tb5_body<MRT, K, REC, ST>(a, tb, blockIdx.x, blockIdx.y, xs_mem, s_tab);
+    tb5_body<MRT, K, ST>(a, tb, blockIdx.x, blockIdx.y, xs_mem, s_tab);
 }
 
 using Tb5Fn = void (*)(const StepArgs, const Tb5Args);
 
 template <int K, typename ST> Tb5Fn pick_k(bool mrt) {
-    return mrt ? tb5_kernel<true, K, false, ST> : tb5_kernel<false, K, false, ST>;
+    return mrt ? tb5_kernel<true, K, ST> : tb5_kernel<false, K, ST>;
 }
 
 }  // namespace lbtb5
